@@ -1301,6 +1301,10 @@ int prepare_run(const kpm_model *m, int n_sectors, const int32_t *n_up, int K, i
     full |= n_up[s] < 0;
   }
   fill_bonds(m, &run->bonds);
+  run->fx_unit = run->bonds.n_groups > 0 ? fixed_unit(run->bonds) : weighted_unit(m->n_bonds);
+  // fixed-point vectors where they round no more than FP64 ones (kpm_fixed.cuh)
+  const bool fixed_point = precision == KPM_FP64 && vectors == kVecRademacher && knobs.fixed != 0 &&
+                           run->fx_unit >= kFxMinUnit;
   // neighbour lists for cooperative layouts with grouped couplings (CPL 1 or 2)
   run->list_stride = 0;
   run->fixed = false;
@@ -1316,7 +1320,7 @@ int prepare_run(const kpm_model *m, int n_sectors, const int32_t *n_up, int K, i
       run->lay.cpl = 2;
       run->lay.gpw = 2;
     }
-    run->fixed = knobs.fixed != 0 && precision == KPM_FP64 && vectors == kVecRademacher;
+    run->fixed = fixed_point;
     // header word, then each group's entries (FP32, fixed point: padded to whole gather batches)
     auto stride_of = [&](int B) {
       int stride = 1;
@@ -1366,7 +1370,7 @@ int prepare_run(const kpm_model *m, int n_sectors, const int32_t *n_up, int K, i
   run->weighted = false;
   if (knobs.lists != 0 && knobs.weighted != 0 && run->bonds.n_groups == 0 && m->n_bonds > 0 &&
       run->lay.G >= 2 && run->lay.cpl <= 2 &&
-      (precision == KPM_FP32 || (vectors == kVecRademacher && knobs.fixed != 0))) {
+      (precision == KPM_FP32 || fixed_point)) {
     run->wr.stride = weighted_stride(m->n_bonds);
     if ((uint64_t)rows * run->wr.stride * sizeof(uint4) <= kWeightedMaxBytes) {
       run->weighted = true;
@@ -1456,10 +1460,8 @@ int prepare_run(const kpm_model *m, int n_sectors, const int32_t *n_up, int K, i
     run->n_cd = (int)(run->cd_chunks.size() / 3);
     run->cd_chunks.insert(run->cd_chunks.end(), ranges.begin(), ranges.end());
   }
-  run->small = precision == KPM_FP64 && vectors == kVecRademacher && knobs.fixed != 0 &&
-               knobs.small != 0 && small_applies(m, n_sectors, n_up);
+  run->small = fixed_point && knobs.small != 0 && small_applies(m, n_sectors, n_up);
   if (run->small) KPM_TRY(prepare_small(m, run));
-  run->fx_unit = run->bonds.n_groups > 0 ? fixed_unit(run->bonds) : weighted_unit(m->n_bonds);
   fill_pass_masks(&run->bonds, run->lay.G);
   run->NQ = run->plan.any_full ? 6 : 2;
   KPM_REQUIRE((uint64_t)(run->plan.total_rows + 1) * (run->lay.Rp / run->lay.vec_width) < (1ull << 32),

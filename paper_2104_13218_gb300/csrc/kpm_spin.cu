@@ -662,7 +662,9 @@ int prepare_spin(const kpm_spin_model *m, int n_sectors, const int32_t *Q, int R
     rows += std::max<int64_t>(0, kpm_spin_sector_dim(m->n_sites, m->two_s, Q[i]));
   RowLayout &lay = run->lay;
   run->wr.stride = weighted_stride(2 * m->n_bonds);
+  run->wr.unit = weighted_unit(2 * m->n_bonds);
   run->weighted = lists && lay.cpl <= 2 && m->n_bonds > 0 &&
+                  (precision == KPM_FP32 || run->wr.unit >= kFxMinUnit) &&
                   (uint64_t)(rows + 1) * (lay.Rp / lay.vec_width) < (1ull << 32) &&
                   (uint64_t)rows * run->wr.stride * sizeof(uint4) <= kWeightedMaxBytes;
   run->fixed = run->weighted && precision == KPM_FP64;
@@ -686,7 +688,6 @@ int prepare_spin(const kpm_spin_model *m, int n_sectors, const int32_t *Q, int R
   WeightedRun &w = run->wr;
   w.full = full;
   w.exact_dots = true;
-  w.unit = weighted_unit(2 * m->n_bonds);
   // with lists one all-zero row follows the last state
   run->vec_bytes = align256((size_t)(run->plan.total_rows + (run->weighted ? 1 : 0)) * lay.Rp * lay.elem);
   return KPM_OK;

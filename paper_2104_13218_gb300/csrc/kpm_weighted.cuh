@@ -12,6 +12,7 @@
 
 #include <algorithm>
 
+#include "kpm_fixed.cuh"
 #include "kpm_internal.h"
 
 namespace kpm {
@@ -43,10 +44,11 @@ struct WeightedRun {
   bool exact_dots = false;        // FP32: dot products as if summed in FP64
 };
 
-// U for rows of at most `entries` neighbours: (entries + 1) 16 U <= 2^61 keeps the
-// middle limbs of a row's sum below 2^63 (kpm_fixed.cuh).
+// U for rows of at most `entries` neighbours: (entries + 1) 8 U <= 2^62 keeps the
+// middle limbs of a row's sum, that and kFxMaxRow 2^59, below 2^63 (kpm_fixed.cuh).
 inline int64_t weighted_unit(int entries) {
-  return std::min<int64_t>((int64_t)1 << 53, ((int64_t)1 << 61) / (16 * ((int64_t)entries + 1))) - 1;
+  return std::min<int64_t>((int64_t)1 << 54,
+                           ((int64_t)1 << 62) / (kFxRange * ((int64_t)entries + 1))) - 1;
 }
 
 // Step kernel of a run (fixed point for KPM_FP64; at most two chunks per lane).

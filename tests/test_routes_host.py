@@ -1,0 +1,58 @@
+"""The rules that choose a form of the moment loop's step (CPU only)."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+import kpm_workloads as W
+from paper_2104_13218_gb300 import _lib
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+
+@pytest.fixture(scope="module")
+def route(tmp_path_factory):
+    cxx = shutil.which("g++")
+    if cxx is None:
+        pytest.skip("no host C++ compiler")
+    _lib.lib()  # builds libkpm.so if needed
+    libdir = os.path.join(ROOT, "paper_2104_13218_gb300", "_build")
+    exe = str(tmp_path_factory.mktemp("route") / "route_dump")
+    cuda_inc = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
+    subprocess.run([cxx, "-O1", "-std=c++17", "-I" + os.path.join(ROOT, "include"),
+                    "-I" + os.path.join(ROOT, "paper_2104_13218_gb300", "csrc"), "-I" + cuda_inc,
+                    os.path.join(HERE, "host", "route_dump.cpp"), "-o", exe, "-L" + libdir, "-lkpm",
+                    "-Wl,-rpath," + libdir], check=True)
+
+    def run(model, n_up, R, precision="fp64", K=200):
+        bonds = [f"{i} {j} {J!r}" for i, j, J in zip(model.bi, model.bj, map(float, model.J))]
+        text = " ".join(map(str, [model.n_sites, R, K, int(precision == "fp32"), len(n_up), *n_up,
+                                  len(bonds), *bonds]))
+        out = subprocess.run([exe], input=text, check=True, capture_output=True, text=True).stdout.split()
+        assert out[0] == "0"
+        return {k: int(v) for k, v in zip(out[1::2], out[2::2])}
+
+    return run
+
+
+# A step in fixed point rounds a component by 0.29/U in the root mean square, one with
+# FP64 vectors by 2^-53.8 .. 2^-54.05 (both in units of 1/sqrt(D)): no model may be given a
+# unit at which the first is larger.  One and two groups, and couplings of their own,
+# from few to the most bonds, with and without the small-sector kernel.
+@pytest.mark.parametrize("n,k", [(12, 6), (18, 9), (23, 11)])
+def test_fixed_point_rounds_no_more_than_fp64(route, n, k):
+    pairs = [(i, j) for j in range(n) for i in range(j)]
+    seen = set()
+    for count in (1, 12, 20, 40, 44, 51, 52, 66, 84, 101, 102, 120, 153, 253):
+        if count > len(pairs):
+            continue
+        for kind in ("one", "two", "own"):
+            J = {"one": lambda b: 1.0, "two": lambda b: 1.0 + (b % 2), "own": lambda b: 1.0 + 0.01 * b}[kind]
+            model = W._model(kind, n, [(i, j, J(b)) for b, (i, j) in enumerate(pairs[:count])])
+            r = route(model, [k], 16)
+            if r["small"] or r["fixed"]:
+                assert 0.29 / r["unit"] <= 2 ** -54.05, (kind, count, r)
+                seen.add(kind)
+    assert seen == {"one", "two", "own"}
