@@ -81,7 +81,7 @@ struct SmallRun {
   const FxCoef *coef = nullptr;
   int n_ent = 0, n_coef = 0;
   const int *block_sector = nullptr, *block_column = nullptr;
-  double *part = nullptr;  // [sector][R][S][2]
+  __int128 *part = nullptr;  // [sector][R][S][2]
 };
 
 // Everything one forward run needs on the device.

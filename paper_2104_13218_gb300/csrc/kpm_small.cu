@@ -43,7 +43,7 @@ struct SmallArgs {
   const FxCoef *coef;   // [n_sectors][n_coef]: 2/a J_g/2 per group, or per bond
   int n_coef;
   const int *block_sector, *block_column;  // largest sectors first
-  double *part;         // [sector][R][S][2]
+  i128 *part;           // [sector][R][S][2], in units of 2^kFxSumShift
   int S, R, n_groups;
   int64_t unit;
   uint64_t seed, r0;
@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) small_run_kernel(const __gri
   }
   __syncthreads();
   unsigned top = 0;
-  double *out = a.part + ((size_t)sec * a.R + col) * a.S * 2;
+  i128 *out = a.part + ((size_t)sec * a.R + col) * a.S * 2;
   for (int n = 0; n < a.S; ++n) {
     FxDot xx, yx;
     const unsigned xs = smem_address(x), zs = smem_address(z);
@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) small_run_kernel(const __gri
     if (warp == n % nw) {
       i128 w[2] = {slot[lane], slot[32 + lane]};
       const i128 r = warp_sums<2>(w);
-      if ((lane & 15) == 0) out[(size_t)n * 2 + (lane >> 4)] = i128_to_double(r) * sd.fx_scale;
+      if ((lane & 15) == 0) out[(size_t)n * 2 + (lane >> 4)] = fx_sum_units(r);
     }
     long long *swap = x;
     x = z;
@@ -259,35 +259,37 @@ __global__ void __launch_bounds__(kSmallThreads, 1) small_run_kernel(const __gri
 }
 
 // sums[step][sector][q] over the vectors (and, for the whole space, over its
-// sectors) in order, and (sums_r) every vector's.  Sector i of the run is made of
-// the blocks' sectors first[i] .. first[i + 1] - 1.
+// sectors), and (sums_r) every vector's.  Sector i of the run is made of the blocks'
+// sectors first[i] .. first[i + 1] - 1.  The sums are exact integers, rounded once: a
+// vector's is below 2^16 states times 2^108 (U <= 2^54, norm 1) in units of 2^20, and with
+// 512 vectors and (2M)^2 <= 2^8 below 2^122.
 template <int NQ>
-__global__ void small_sums_kernel(const double *part, const int *first, const SectorDev *sub,
+__global__ void small_sums_kernel(const i128 *part, const int *first, const SectorDev *sub, int n_sites,
                                   double *sums, double *sums_r, int S, int ns, int R) {
   const int total = S * ns * 2;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-    const int q = i % 2, sec = (i / 2) % ns, n = i / (2 * ns);
-    double v0 = 0.0, v1 = 0.0, v2 = 0.0;
-    for (int k = first[sec]; k < first[sec + 1]; ++k) {
-      const double M = sub[k].Mval;
-      double v = 0.0;
-      for (int r = 0; r < R; ++r) {
-        const double p = part[(((size_t)k * R + r) * S + n) * 2 + q];
+    const int q = i % 2, n = (i / 2) % S, sec = i / (2 * S);
+    const double scale = sub[first[sec]].fx_scale * (1 << kFxSumShift);
+    i128 v0 = 0, v1 = 0, v2 = 0;
+    for (int r = 0; r < R; ++r) {
+      i128 v = 0;
+      for (int k = first[sec]; k < first[sec + 1]; ++k) {
+        const i128 p = part[(((size_t)k * R + r) * S + n) * 2 + q];
         v += p;
-        if (sums_r != nullptr) {
-          double *o = sums_r + (((size_t)n * ns + sec) * R + r) * 2 + q;
-          *o = k == first[sec] ? p : *o + p;
+        if (NQ == 6) {
+          const int m = 2 * sub[k].n_up - n_sites;
+          v1 += p * m;
+          v2 += p * (m * m);
         }
       }
       v0 += v;
-      v1 += M * v;
-      v2 += M * M * v;
+      if (sums_r != nullptr) sums_r[(((size_t)n * ns + sec) * R + r) * 2 + q] = i128_to_double(v) * scale;
     }
     double *o = sums + ((size_t)n * ns + sec) * NQ;
-    o[q] = v0;
+    o[q] = i128_to_double(v0) * scale;
     if (NQ == 6) {
-      o[2 + q] = v1;
-      o[4 + q] = v2;
+      o[2 + q] = i128_to_double(v1) * scale * 0.5;
+      o[4 + q] = i128_to_double(v2) * scale * 0.25;
     }
   }
 }
@@ -343,7 +345,7 @@ size_t small_bytes(const MomentsRun &r) {
          (r.per_vector ? align256((size_t)r.S * r.plan.n_sectors * R * 16) : 0) + align256(rows * 4) +
          align256(rows * sizeof(FxCoef)) + align256(rows * 8) + align256(rows * small_entries(r.bonds) * 4) +
          align256(ns * std::max(kMaxGroups, r.bonds.n_bonds) * sizeof(FxCoef)) +
-         align256((r.plan.n_sectors + 1) * 4) + 2 * align256(ns * R * 4) + align256(ns * R * r.S * 16);
+         align256((r.plan.n_sectors + 1) * 4) + 2 * align256(ns * R * 4) + align256(ns * R * r.S * 2 * sizeof(i128));
 }
 
 int setup_small(MomentsRun &r, const std::vector<SectorDev> &sec, Arena &arena, cudaStream_t s) {
@@ -373,7 +375,7 @@ int setup_small(MomentsRun &r, const std::vector<SectorDev> &sec, Arena &arena, 
   m.diag = arena.take<FxCoef>(rows);
   m.ent = arena.take<uint32_t>(rows * m.n_ent);
   m.code = arena.take<uint64_t>(rows);
-  m.part = arena.take<double>(ns * R * r.S * 2);
+  m.part = arena.take<i128>(ns * R * r.S * 2);
   if (r.per_vector) r.sums_r = arena.take<double>((size_t)r.S * r.plan.n_sectors * R * 2);
   KPM_REQUIRE(m.head && m.diag && m.ent && m.code && m.part &&
                   (!r.per_vector || r.sums_r), KPM_ENOMEM, "workspace too small for the small-sector run");
@@ -457,9 +459,11 @@ int launch_small(const MomentsRun &r, uint64_t seed, uint64_t r0, cudaStream_t s
   const int grid = std::min(2048, (total + 63) / 64);
   double *sums_r = r.per_vector ? r.sums_r : nullptr;
   if (r.NQ == 6)
-    small_sums_kernel<6><<<grid, 64, 0, s>>>(m.part, m.first, m.tb.sectors, r.sums, sums_r, r.S, ns, r.lay.R);
+    small_sums_kernel<6><<<grid, 64, 0, s>>>(m.part, m.first, m.tb.sectors, r.plan.N, r.sums, sums_r, r.S,
+                                             ns, r.lay.R);
   else
-    small_sums_kernel<2><<<grid, 64, 0, s>>>(m.part, m.first, m.tb.sectors, r.sums, sums_r, r.S, ns, r.lay.R);
+    small_sums_kernel<2><<<grid, 64, 0, s>>>(m.part, m.first, m.tb.sectors, r.plan.N, r.sums, sums_r, r.S,
+                                             ns, r.lay.R);
   KPM_CUDA(cudaGetLastError());
   count_launches(1);
   return KPM_OK;

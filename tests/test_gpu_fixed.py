@@ -275,3 +275,18 @@ def test_small_sectors_single_product():
     for i, k in enumerate((3, 2)):
         ref = c_oracle.moments(6, bi, bj, J, k, 2.4, -0.6, 2, 3, 5)["mu"]
         assert np.abs(got["mu"][i] - ref).max() <= 1e-14
+
+
+# ---------------------------------------------------------------- M-weighted sums of the whole space
+# With -J and -b in place of J and b every v_n becomes (-1)^n v_n, bit for bit, so
+# the odd moments change sign and nothing else: what is left of their sum is a bias of the sums.
+# Tolerance: four roundings of a double in [0.5, 1).  Units near the lowest, rows with
+# unused columns; lists with matrix elements, with groups, and small sectors.
+@pytest.mark.parametrize("n,count,R", [(17, 100, 3), (17, -48, 5), (12, 60, 3)])
+def test_weighted_sums_have_no_bias(n, count, R):
+    bi, bj, J = _bonds(n, abs(count)).arrays()
+    J = J if count > 0 else np.ones_like(J)
+    got = [kpm.moments(kpm.CModel(n, bi, bj, s * J), [-1], 12, R, 5, a=[30.0], b=[0.5 * s]) for s in (1, -1)]
+    for q in ("mu", "mu_M", "mu_M2"):
+        assert np.abs(got[0][q][0, 1::2] + got[1][q][0, 1::2]).max() <= 4.5e-16, q
+        assert np.abs(got[0][q][0, 0::2] - got[1][q][0, 0::2]).max() <= 4.5e-16, q
