@@ -578,6 +578,8 @@ struct WeightedListArgs {
   TablesDev tb;
   int stride;
   uint32_t crow, zero_chunk;
+  const int64_t *couplings;  // fixed point: [n_sectors][n_bonds] J/a, and
+  const int64_t *c0;         // [n_sectors] the diagonal without anti-aligned bonds, in 2^-59
   int *flag;
 };
 
@@ -596,7 +598,7 @@ __global__ void __launch_bounds__(32)
       const uint64_t s = sd.n_up < 0 ? (uint64_t)(row - sd.row0)
                                      : sector_unrank(tile.rank0 + u, sd.n_up, tile.b_last, hb, a.tb);
       uint4 *L = a.lists + (size_t)row * a.stride;
-      double d = bd.J_quarter_sum, sum = 0.0;
+      int64_t d = FIXED ? a.c0[tile.sector] : 0, sum = 0;
       float dsum = 0.f;
       uint32_t e = 1;
       for (int b = 0; b < bd.n_bonds; ++b) {
@@ -607,10 +609,10 @@ __global__ void __launch_bounds__(32)
         const uint32_t rk = sd.n_up < 0 ? (uint32_t)f : sector_rank(f, a.tb);
         const uint32_t chunk = ((uint32_t)sd.row0 + rk) * a.crow;
         if (FIXED) {
-          const double c = A * 0.5 * bd.J[b];
-          d -= 0.5 * bd.J[b];
-          sum += fabs(c);
-          const FxCoef k = fx_coef_device(c, out_of_range);
+          const int64_t c = __ldg(a.couplings + (size_t)tile.sector * bd.n_bonds + b);
+          d -= c;
+          sum += llabs(c) >> 8;
+          const FxCoef k = fx_limbs_of(c);
           L[e++] = make_uint4(chunk, (unsigned)k.h, k.l, 0);
         } else {
           dsum += (float)(0.5 * bd.J[b]);
@@ -621,9 +623,9 @@ __global__ void __launch_bounds__(32)
       while ((e - 1) % kWeightedBatch != 0) L[e++] = make_uint4(a.zero_chunk, 0, 0, 0);
       const int m2 = sd.n_up < 0 ? 2 * __popcll(s) - bd.n_sites : 2 * sd.n_up - bd.n_sites;
       if (FIXED) {
-        const double c = A * (d - sd.b);
-        const FxCoef k = fx_coef_device(c, out_of_range);
-        out_of_range |= !(sum + fabs(c) <= kFxMaxRow);
+        // (where the sum is in range, d cannot have overflowed)
+        const FxCoef k = fx_limbs_of(d);
+        out_of_range |= sum + (llabs(d) >> 8) > kFxRowUnits || llabs(d) > kFxCoefUnits;
         L[0] = make_uint4(cnt, (unsigned)k.h, k.l, (unsigned)m2);
       } else {
         const float ad = (float)A * (((float)bd.J_quarter_sum - dsum) - (float)sd.b);
@@ -1041,7 +1043,7 @@ struct AssembleRArgs {
   const double *sums_r;  // [S][n_sectors][R][2]
   const SectorDev *sectors;
   double *mu_r;
-  int n_sectors, K, R;
+  int n_sectors, K, R, subtracted;
 };
 
 __global__ void assemble_r_kernel(const __grid_constant__ AssembleRArgs a) {
@@ -1054,7 +1056,7 @@ __global__ void assemble_r_kernel(const __grid_constant__ AssembleRArgs a) {
     const int step = n / 2, q = n & 1;
     const double raw = a.sums_r[(((int64_t)step * a.n_sectors + sec) * a.R + r) * 2 + q];
     const double base = a.sums_r[((int64_t)sec * a.R + r) * 2 + q];  // mu_0 or mu_1 of vector r
-    const double val = step == 0 ? raw : 2.0 * raw - base;
+    const double val = step == 0 || a.subtracted ? raw : 2.0 * raw - base;
     a.mu_r[((int64_t)a.sectors[sec].out_index * a.R + r) * a.K + n] = val;
   }
 }
@@ -1134,6 +1136,7 @@ struct AssembleArgs {
   double *mu, *mu_M, *mu_M2;
   int *flag;
   int n_sectors, K, NQ;
+  int subtracted;  // the sums of the later steps are 2 <v_n|v_n> - <v_0|v_0> already
   double inv_R;
 };
 
@@ -1152,7 +1155,7 @@ __global__ void assemble_kernel(const __grid_constant__ AssembleArgs a) {
       if (full || q == 0) {
         const int qq = 2 * q + (odd ? 1 : 0);
         const double raw = a.sums[((int64_t)step * a.n_sectors + sec) * a.NQ + qq] * a.inv_R;
-        if (step == 0) {
+        if (step == 0 || a.subtracted) {
           val = raw;
         } else {
           const double base = a.sums[(int64_t)sec * a.NQ + qq] * a.inv_R;  // mu_0 or mu_1
@@ -1163,7 +1166,7 @@ __global__ void assemble_kernel(const __grid_constant__ AssembleArgs a) {
         const int qq = odd ? 1 : 0;
         const double raw = a.sums[((int64_t)step * a.n_sectors + sec) * a.NQ + qq] * a.inv_R;
         const double base = a.sums[(int64_t)sec * a.NQ + qq] * a.inv_R;
-        const double m0 = step == 0 ? raw : 2.0 * raw - base;
+        const double m0 = step == 0 || a.subtracted ? raw : 2.0 * raw - base;
         const double M = a.sectors[sec].Mval;
         val = (q == 1 ? M : M * M) * m0;
       }
@@ -1486,7 +1489,8 @@ size_t stepped_bytes(const MomentsRun &r) {
   const bool lists = r.list_stride > 0;
   const size_t weighted =
       r.weighted ? align256((size_t)r.plan.total_rows * r.wr.stride * sizeof(uint4)) +
-                       align256((size_t)r.plan.n_sectors * sizeof(double))
+                       align256((size_t)r.plan.n_sectors * sizeof(double)) +
+                       align256((size_t)r.plan.n_sectors * (r.bonds.n_bonds + 1) * sizeof(int64_t)) + 256
                  : 0;
   size_t coef = 0;
   if (lists)
@@ -1572,9 +1576,9 @@ int upload_coefficients_t(MomentsRun &r, const std::vector<SectorDev> &sec, Aren
 
 int upload_coefficients(MomentsRun &r, const std::vector<SectorDev> &sec, Arena &arena,
                         cudaStream_t s) {
-  std::vector<FxCoef> diag, grp;
-  r.fixed = r.fixed && fixed_coefficients(r.bonds, sec, &diag, &grp);
   if (r.fixed) {
+    std::vector<FxCoef> diag, grp;
+    fixed_tables(r.bonds, r.fx_couplings, r.fx_c0, &diag, &grp);
     const std::vector<FxCoef> *src[4] = {&diag, nullptr, &grp, nullptr};
     for (int w = 0; w < 4; ++w) {
       r.coef[w] = arena.take<char>(coef_bytes(r, w));
@@ -1629,6 +1633,13 @@ int setup_weighted(MomentsRun &r, const std::vector<SectorDev> &sec, Arena &aren
   la.crow = (uint32_t)(r.lay.Rp / r.lay.vec_width);
   la.zero_chunk = (uint32_t)r.plan.total_rows * la.crow;
   la.flag = r.flag;
+  la.couplings = la.c0 = nullptr;
+  if (r.fixed) {
+    PackedUpload up(arena, s);
+    KPM_TRY(up.add(r.fx_couplings, &la.couplings));
+    KPM_TRY(up.add(r.fx_c0, &la.c0));
+    KPM_TRY(up.send());
+  }
   const int grid = (int)std::min<int64_t>((int64_t)r.plan.tiles.size(), (int64_t)32 * sm_count());
   if (r.fixed)
     build_weighted_lists_kernel<true><<<grid, 32, 0, s>>>(la, r.bonds);
@@ -1643,8 +1654,10 @@ int setup_weighted(MomentsRun &r, const std::vector<SectorDev> &sec, Arena &aren
 
 int setup_run(MomentsRun &r, const double *a, const double *b, Arena &arena, cudaStream_t s,
               const int *out_index) {
+  if ((r.fixed || r.small) &&
+      !fixed_couplings(r.bonds, r.plan, a, b, &r.fx_couplings, &r.fx_c0))
+    r.fixed = r.small = false;  // out of the fixed-point range: the run in FP64
   if (r.weighted && r.precision == KPM_FP64) r.weighted = r.fixed;
-  const Arena start = arena;
   if (!r.small) {
     r.vA = arena.take<char>(r.vec_bytes);
     r.vB = arena.take<char>(r.vec_bytes);
@@ -1682,17 +1695,11 @@ int setup_run(MomentsRun &r, const double *a, const double *b, Arena &arena, cud
     sec[i].pad2 = 0;
   }
   KPM_TRY(upload_tables(r.plan, sec, arena, s, &r.tb));
-  if (r.small) {
-    KPM_TRY(setup_small(r, sec, arena, s));
-    if (r.small) return KPM_OK;
-    arena = start;  // out of the fixed-point range: the run in FP64
-    r.fixed = false;
-    return setup_run(r, a, b, arena, s, out_index);
-  }
+  if (r.small) return setup_small(r, sec, arena, s);
   if (r.list_stride > 0) {
     r.lists = arena.take<uint32_t>((size_t)r.plan.total_rows * r.list_stride);
     KPM_REQUIRE(r.lists != nullptr, KPM_ENOMEM, "workspace too small for the neighbour lists");
-    KPM_TRY(upload_coefficients(r, sec, arena, s));  // settles r.fixed
+    KPM_TRY(upload_coefficients(r, sec, arena, s));
     ListArgs la;
     la.lists = r.lists;
     la.tb = r.tb;
@@ -1946,6 +1953,7 @@ int launch_assemble(const MomentsRun &r, double *mu, double *mu_M, double *mu_M2
     ar.n_sectors = r.plan.n_sectors;
     ar.K = r.K;
     ar.R = r.lay.R;
+    ar.subtracted = r.small;
     const int64_t tot = (int64_t)r.plan.n_sectors * r.lay.R * r.K;
     assemble_r_kernel<<<(int)std::min<int64_t>(4096, (tot + 255) / 256), 256, 0, s>>>(ar);
     KPM_CUDA(cudaGetLastError());
@@ -1961,6 +1969,7 @@ int launch_assemble(const MomentsRun &r, double *mu, double *mu_M, double *mu_M2
   a.n_sectors = r.plan.n_sectors;
   a.K = r.K;
   a.NQ = r.NQ;
+  a.subtracted = r.small;
   a.inv_R = 1.0 / r.lay.R;
   const int total = r.plan.n_sectors * r.K;
   assemble_kernel<<<(total + 255) / 256, 256, 0, s>>>(a);

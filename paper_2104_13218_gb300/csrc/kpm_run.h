@@ -128,6 +128,7 @@ struct MomentsRun {
   // coefficients or, during the run, the components leave the range.
   bool fixed = false;
   int64_t fx_unit = 0;             // U
+  std::vector<int64_t> fx_couplings, fx_c0;  // fixed_couplings of the run
   // Lists with matrix elements (kpm_weighted.cuh): cooperative layouts whose
   // couplings have too many values for groups, in FP32 and in fixed point.
   bool weighted = false;
@@ -228,7 +229,7 @@ constexpr int64_t kSmallMaxDim = 13500;
 bool small_applies(const kpm_model *m, int n_sectors, const int32_t *n_up);
 int prepare_small(const kpm_model *m, MomentsRun *run);
 size_t small_bytes(const MomentsRun &r);
-// Carves and fills the run's buffers; clears r.small when a coupling is out of range.
+// Carves and fills the run's buffers.
 int setup_small(MomentsRun &r, const std::vector<SectorDev> &sec, Arena &arena, cudaStream_t s);
 // Random vectors, all products and their sums.
 int launch_small(const MomentsRun &r, uint64_t seed, uint64_t r0, cudaStream_t s);
@@ -244,8 +245,15 @@ int launch_small(const MomentsRun &r, uint64_t seed, uint64_t r0, cudaStream_t s
 #endif
 __host__ __device__ constexpr int fixed_batch(int cpl) { return KPM_FIXED_BATCH / cpl; }
 int64_t fixed_unit(const BondsDev &b);
-bool fixed_coefficients(const BondsDev &bd, const std::vector<SectorDev> &sec,
-                        std::vector<FxCoef> *diag, std::vector<FxCoef> *grp);
+// Coefficients of 2H/a and 2(H - b)/a in units of 2^-59: per sector J/a of every group
+// (or bond), and the diagonal of a state without anti-aligned bonds, of which each
+// anti-aligned bond takes its J/a away.  False when one is out of range.
+bool fixed_couplings(const BondsDev &bd, const Plan &p, const double *a, const double *b,
+                     std::vector<int64_t> *couplings, std::vector<int64_t> *c0);
+// The list kernel's tables: the diagonal for every combination of anti-aligned bond
+// counts, marked where it is out of range, and the groups' couplings.
+void fixed_tables(const BondsDev &bd, const std::vector<int64_t> &couplings,
+                  const std::vector<int64_t> &c0, std::vector<FxCoef> *diag, std::vector<FxCoef> *grp);
 void *fixed_kernel_ptr(int cpl, bool full);
 int launch_fixed_step(const MomentsRun &run, const void *x, void *zy, int first, double *partials,
                       const double *prev_partials, double *prev_sums, int sum_parts, int *queue,

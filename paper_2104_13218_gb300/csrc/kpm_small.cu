@@ -54,6 +54,9 @@ struct SmallArgs {
 struct SmallListArgs {
   TablesDev tb;
   SmallLists l;
+  const int64_t *coef;  // [n_sectors][n_coef] J/a, and
+  const int64_t *c0;    // [n_sectors] the diagonal without anti-aligned bonds, in units of 2^-59
+  int n_coef;
   int *flag;
 };
 
@@ -64,7 +67,8 @@ __global__ void __launch_bounds__(kThreads)
   for (int t = blockIdx.x; t < a.tb.n_tiles; t += gridDim.x) {
     const Tile tile = a.tb.tiles[t];
     const SectorDev sd = a.tb.sectors[tile.sector];
-    const double A = 2.0 * sd.inv_a;
+    const int64_t *coef = a.coef + (size_t)tile.sector * a.n_coef;
+    const int64_t c0 = a.c0[tile.sector];
     uint32_t hb = tile.b_first;
     for (uint32_t i = threadIdx.x; i < tile.count; i += kThreads) {
       const int64_t row = tile.row0 + i;
@@ -72,7 +76,7 @@ __global__ void __launch_bounds__(kThreads)
       const uint64_t s = sd.n_up < 0 ? (uint64_t)u
                                      : sector_unrank(tile.rank0 + i, sd.n_up, tile.b_last, hb, a.tb);
       uint32_t *E = a.l.ent + (size_t)sd.row0 * a.l.n_ent + u;
-      double d = bd.J_quarter_sum, sum = 0.0;
+      int64_t d = c0, sum = 0;
       uint32_t head = 0, pair = 0;
       size_t e = 0;
       const int ng = GROUPED ? bd.n_groups : 1;
@@ -86,8 +90,9 @@ __global__ void __launch_bounds__(kThreads)
           if (tt == 0 || tt == m) continue;
           const uint64_t f = s ^ m;
           const uint32_t rk = sd.n_up < 0 ? (uint32_t)f : sector_rank(f, a.tb);
-          d -= 0.5 * bd.J[b];
-          sum += fabs(A * 0.5 * bd.J[b]);
+          const int64_t c = __ldg(coef + (GROUPED ? g : k));
+          d -= c;
+          sum += llabs(c) >> 8;
           if (!GROUPED) {
             E[(e++) * sd.dim] = rk | ((uint32_t)b << 16);
           } else if (cnt & 1) {
@@ -100,11 +105,11 @@ __global__ void __launch_bounds__(kThreads)
         if (GROUPED && (cnt & 1)) E[(e++) * sd.dim] = pair | ((uint32_t)sd.dim << 16);
         head |= cnt << (8 * g);
       }
-      const double c = A * (d - sd.b);
-      out_of_range |= !(sum + fabs(c) <= kFxMaxRow);
+      // (where the sum is in range, d cannot have overflowed)
+      out_of_range |= sum + (llabs(d) >> 8) > kFxRowUnits || llabs(d) > kFxCoefUnits;
       a.l.head[row] = head;
       a.l.code[row] = s;
-      a.l.diag[row] = fx_coef_device(c, out_of_range);
+      a.l.diag[row] = fx_limbs_of(d);
     }
   }
   if (out_of_range) atomicOr(a.flag, kFlagRange);
@@ -259,37 +264,53 @@ __global__ void __launch_bounds__(kSmallThreads, 1) small_run_kernel(const __gri
 }
 
 // sums[step][sector][q] over the vectors (and, for the whole space, over its
-// sectors), and (sums_r) every vector's.  Sector i of the run is made of the blocks'
-// sectors first[i] .. first[i + 1] - 1.  The sums are exact integers, rounded once: a
-// vector's is below 2^16 states times 2^108 (U <= 2^54, norm 1) in units of 2^20, and with
-// 512 vectors and (2M)^2 <= 2^8 below 2^122.
+// sectors), and (sums_r) every vector's: of step 0 the dot products, of step n > 0
+// already the moments' 2 <v_n|v_n> - <v_0|v_0> and 2 <v_{n+1}|v_n> - <v_1|v_0>, which FP64
+// would round to 2^-54 of terms near 1 where the difference is some 1/sqrt(D).  Sector i
+// of the run is made of the blocks' sectors first[i] .. first[i + 1] - 1.  The sums are exact
+// integers, rounded once: a vector's is below 2^16 states times 2^108 (U <= 2^54, norm 1) in
+// units of 2^20, and doubled, with 512 vectors and (2M)^2 <= 2^8, below 2^123.
+// A warp takes one step of one sector, its lanes the vectors.
+constexpr int kSumsThreads = 128;
 template <int NQ>
-__global__ void small_sums_kernel(const i128 *part, const int *first, const SectorDev *sub, int n_sites,
-                                  double *sums, double *sums_r, int S, int ns, int R) {
-  const int total = S * ns * 2;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-    const int q = i % 2, n = (i / 2) % S, sec = i / (2 * S);
-    const double scale = sub[first[sec]].fx_scale * (1 << kFxSumShift);
-    i128 v0 = 0, v1 = 0, v2 = 0;
-    for (int r = 0; r < R; ++r) {
-      i128 v = 0;
-      for (int k = first[sec]; k < first[sec + 1]; ++k) {
-        const i128 p = part[(((size_t)k * R + r) * S + n) * 2 + q];
-        v += p;
-        if (NQ == 6) {
-          const int m = 2 * sub[k].n_up - n_sites;
-          v1 += p * m;
-          v2 += p * (m * m);
+__global__ void __launch_bounds__(kSumsThreads)
+    small_sums_kernel(const i128 *part, const int *first, const SectorDev *sub, int n_sites, double *sums,
+                      double *sums_r, int S, int ns, int R) {
+  const int lane = threadIdx.x & 31;
+  for (int i = (blockIdx.x * kSumsThreads + threadIdx.x) / 32; i < S * ns; i += gridDim.x * kSumsThreads / 32) {
+    const int n = i % S, sec = i / S;
+    const int k0 = first[sec], k1 = first[sec + 1];
+    const double scale = sub[k0].fx_scale * (1 << kFxSumShift);
+    i128 acc[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) acc[q] = 0;
+    for (int r = lane; r < R; r += 32) {
+      i128 v[2] = {0, 0};
+      for (int k = k0; k < k1; ++k) {
+        const i128 *mine = part + ((size_t)k * R + r) * S * 2;
+        const int m = NQ == 6 ? 2 * sub[k].n_up - n_sites : 0;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const i128 p = n == 0 ? mine[q] : 2 * mine[2 * n + q] - mine[q];
+          v[q] += p;
+          if (NQ == 6) {
+            acc[(2 + q) % NQ] += p * m;
+            acc[(4 + q) % NQ] += p * (m * m);
+          }
         }
       }
-      v0 += v;
-      if (sums_r != nullptr) sums_r[(((size_t)n * ns + sec) * R + r) * 2 + q] = i128_to_double(v) * scale;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        acc[q] += v[q];
+        if (sums_r != nullptr)
+          sums_r[(((size_t)n * ns + sec) * R + r) * 2 + q] = i128_to_double(v[q]) * scale;
+      }
     }
     double *o = sums + ((size_t)n * ns + sec) * NQ;
-    o[q] = i128_to_double(v0) * scale;
-    if (NQ == 6) {
-      o[2 + q] = i128_to_double(v1) * scale * 0.5;
-      o[4 + q] = i128_to_double(v2) * scale * 0.25;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      const i128 w = warp_sum_i128(acc[q]);
+      if (lane == 0) o[q] = i128_to_double(w) * scale * (q < 2 ? 1.0 : q < 4 ? 0.5 : 0.25);
     }
   }
 }
@@ -344,7 +365,7 @@ size_t small_bytes(const MomentsRun &r) {
          align256((size_t)2 * r.S * 4) + 256 +
          (r.per_vector ? align256((size_t)r.S * r.plan.n_sectors * R * 16) : 0) + align256(rows * 4) +
          align256(rows * sizeof(FxCoef)) + align256(rows * 8) + align256(rows * small_entries(r.bonds) * 4) +
-         align256(ns * std::max(kMaxGroups, r.bonds.n_bonds) * sizeof(FxCoef)) +
+         2 * align256(ns * std::max(kMaxGroups, r.bonds.n_bonds) * sizeof(FxCoef)) + align256(ns * 8) +
          align256((r.plan.n_sectors + 1) * 4) + 2 * align256(ns * R * 4) + align256(ns * R * r.S * 2 * sizeof(i128));
 }
 
@@ -379,16 +400,17 @@ int setup_small(MomentsRun &r, const std::vector<SectorDev> &sec, Arena &arena, 
   if (r.per_vector) r.sums_r = arena.take<double>((size_t)r.S * r.plan.n_sectors * R * 2);
   KPM_REQUIRE(m.head && m.diag && m.ent && m.code && m.part &&
                   (!r.per_vector || r.sums_r), KPM_ENOMEM, "workspace too small for the small-sector run");
-  // couplings of 2H/a; a one-state sector has none
-  std::vector<FxCoef> c(ns * m.n_coef, FxCoef{0, 0});
-  for (size_t i = 0; i < ns; ++i)
-    for (int k = 0; k < m.n_coef && p.dim[i] > 1; ++k) {
-      const double v = 2.0 * sub[i].inv_a * 0.5 * (bd.n_groups > 0 ? bd.gJ[k] : bd.J[k]);
-      if (!(std::fabs(v) <= kFxMaxCoef)) {
-        r.small = false;
-        return KPM_OK;
+  // couplings of 2H/a, those of the run's sector
+  std::vector<FxCoef> c(ns * m.n_coef);
+  std::vector<int64_t> units(ns * m.n_coef), c0(ns);
+  for (int i = 0; i < r.plan.n_sectors; ++i)
+    for (int j = first[i]; j < first[i + 1]; ++j) {
+      c0[j] = r.fx_c0[i];
+      for (int k = 0; k < m.n_coef; ++k) {
+        const int64_t v = r.fx_couplings[(size_t)i * m.n_coef + k];
+        units[(size_t)j * m.n_coef + k] = v;
+        c[(size_t)j * m.n_coef + k] = fx_limbs_of(v);
       }
-      c[i * m.n_coef + k] = fx_coef(v);
     }
   // largest sectors first
   std::vector<int> order(ns), hb, hc;
@@ -402,13 +424,16 @@ int setup_small(MomentsRun &r, const std::vector<SectorDev> &sec, Arena &arena, 
       m.block_dim.push_back((int)p.dim[i]);
     }
   PackedUpload up(arena, s);
+  SmallListArgs la;
   KPM_TRY(up.add(c, &m.coef));
+  KPM_TRY(up.add(units, &la.coef));
+  KPM_TRY(up.add(c0, &la.c0));
   KPM_TRY(up.add(hb, &m.block_sector));
   KPM_TRY(up.add(hc, &m.block_column));
   KPM_TRY(up.add(first, &m.first));
   KPM_TRY(up.send());
-  SmallListArgs la;
   la.tb = m.tb;
+  la.n_coef = m.n_coef;
   la.l = SmallLists{m.head, m.diag, m.ent, m.code, m.n_ent};
   la.flag = r.flag;
   const int grid = (int)std::min<int64_t>((int64_t)p.tiles.size(), (int64_t)8 * sm_count());
@@ -455,15 +480,15 @@ int launch_small(const MomentsRun &r, uint64_t seed, uint64_t r0, cudaStream_t s
   void *args[] = {(void *)&a};
   KPM_CUDA(cudaLaunchKernel(fn, dim3(n_blocks), dim3(threads), args, small_smem(D), s));
   count_launches(1);
-  const int ns = r.plan.n_sectors, total = r.S * ns * 2;
-  const int grid = std::min(2048, (total + 63) / 64);
+  const int ns = r.plan.n_sectors, per_block = kSumsThreads / 32;
+  const int grid = std::min(4096, (r.S * ns + per_block - 1) / per_block);
   double *sums_r = r.per_vector ? r.sums_r : nullptr;
   if (r.NQ == 6)
-    small_sums_kernel<6><<<grid, 64, 0, s>>>(m.part, m.first, m.tb.sectors, r.plan.N, r.sums, sums_r, r.S,
-                                             ns, r.lay.R);
+    small_sums_kernel<6><<<grid, kSumsThreads, 0, s>>>(m.part, m.first, m.tb.sectors, r.plan.N, r.sums,
+                                                       sums_r, r.S, ns, r.lay.R);
   else
-    small_sums_kernel<2><<<grid, 64, 0, s>>>(m.part, m.first, m.tb.sectors, r.plan.N, r.sums, sums_r, r.S,
-                                             ns, r.lay.R);
+    small_sums_kernel<2><<<grid, kSumsThreads, 0, s>>>(m.part, m.first, m.tb.sectors, r.plan.N, r.sums,
+                                                       sums_r, r.S, ns, r.lay.R);
   KPM_CUDA(cudaGetLastError());
   count_launches(1);
   return KPM_OK;

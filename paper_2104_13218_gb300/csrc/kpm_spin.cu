@@ -66,6 +66,7 @@ struct SpinBondsDev {
   double J[kSpinMaxBonds];
   double cp[8], cm[8];   // S^+ and S^- matrix elements for digit q (0 outside the range)
   double s;              // spin
+  int64_t ladder[64];    // fixed point: cp[q] cm[p] 2^58 at [8 q + p] (0: no such element)
   int64_t dpow[kSpinMaxSites];  // d^i (whole-space ranks)
 };
 
@@ -253,6 +254,13 @@ void fill_spin_bonds(const kpm_spin_model *m, SpinBondsDev *b) {
     b->cp[q] = q < m->two_s ? std::sqrt(s * (s + 1) - mm * (mm + 1)) : 0.0;
     b->cm[q] = (q > 0 && q <= m->two_s) ? std::sqrt(s * (s + 1) - mm * (mm - 1)) : 0.0;
   }
+  for (int q = 0; q < m->two_s; ++q)
+    for (int r = 1; r <= m->two_s; ++r) {
+      const double k = (double)(m->two_s - q) * (q + 1) * r * (m->two_s - r + 1);
+      const double h = std::sqrt(k);
+      b->ladder[8 * q + r] = (int64_t)std::ldexp(h, 58) +
+                             (int64_t)std::rint(std::ldexp(std::fma(-h, h, k) / (2.0 * h), 58));
+    }
   int64_t p = 1;
   for (int i = 0; i < kSpinMaxSites; ++i) {
     b->dpow[i] = p;
@@ -289,29 +297,26 @@ __device__ __forceinline__ int64_t spin_rank(uint64_t code, int c, const SpinTab
          (int64_t)__ldg(tb.hi_rank + ((size_t)c << (kSpinBits * tb.H)) + hi);
 }
 
-// Calls f(neighbour row, amplitude) for every off-diagonal element of H in
-// the column of state `code` (row `row`, rank `rank` in its sector) and
-// returns the diagonal element.
+// Calls f(neighbour row, bond, q, p) for every off-diagonal element
+// J/2 cp[q] cm[p] of H in the column of state `code` (row `row`, rank `rank` in its
+// sector).
 template <typename F>
-__device__ __forceinline__ double spin_apply(uint64_t code, int64_t rank, const SpinSectorDev &sd,
+__device__ __forceinline__ void spin_neighbours(uint64_t code, int64_t rank, const SpinSectorDev &sd,
                                              const SpinTablesDev &tb, const SpinBondsDev &bd,
                                              F &&f) {
   const bool full = sd.Q < 0;
   int clo = 0;
   if (!full)
     for (int i = 0; i < tb.L; ++i) clo += digit(code, i);
-  double diag = 0.0;
   for (int b = 0; b < bd.n_bonds; ++b) {
     const int i = bd.bi[b], j = bd.bj[b];
     const int qi = digit(code, i), qj = digit(code, j);
-    const double J = bd.J[b];
-    diag += J * (qi - bd.s) * (qj - bd.s);
     // S^+_i S^-_j (dir 0) and S^-_i S^+_j (dir 1)
 #pragma unroll
     for (int dir = 0; dir < 2; ++dir) {
       const int di = dir == 0 ? 1 : -1;
-      const double amp = 0.5 * J * (dir == 0 ? bd.cp[qi] * bd.cm[qj] : bd.cm[qi] * bd.cp[qj]);
-      if (amp == 0.0) continue;
+      const int q = dir == 0 ? qi : qj, p = dir == 0 ? qj : qi;
+      if (bd.ladder[8 * q + p] == 0) continue;
       const uint64_t nc = (uint64_t)((int64_t)code + (int64_t)di * ((int64_t)1 << (kSpinBits * i)) -
                                      (int64_t)di * ((int64_t)1 << (kSpinBits * j)));
       int64_t nr;
@@ -321,9 +326,24 @@ __device__ __forceinline__ double spin_apply(uint64_t code, int64_t rank, const 
         const int c2 = clo + (i < tb.L ? di : 0) - (j < tb.L ? di : 0);
         nr = spin_rank(nc, c2, tb);
       }
-      f(sd.row0 + nr, amp);
+      f(sd.row0 + nr, b, q, p);
     }
   }
+}
+
+// Calls f(neighbour row, amplitude) for every off-diagonal element and returns the
+// diagonal one.
+template <typename F>
+__device__ __forceinline__ double spin_apply(uint64_t code, int64_t rank, const SpinSectorDev &sd,
+                                             const SpinTablesDev &tb, const SpinBondsDev &bd,
+                                             F &&f) {
+  double diag = 0.0;
+  for (int b = 0; b < bd.n_bonds; ++b)
+    diag += bd.J[b] * (digit(code, bd.bi[b]) - bd.s) * (digit(code, bd.bj[b]) - bd.s);
+  spin_neighbours(code, rank, sd, tb, bd, [&](int64_t nrow, int b, int q, int p) {
+    const double amp = 0.5 * bd.J[b] * (bd.cp[q] * bd.cm[p]);
+    if (amp != 0.0) f(nrow, amp);
+  });
   return diag;
 }
 
@@ -424,12 +444,15 @@ __global__ void __launch_bounds__(kThreads)
 }
 
 // Lists with matrix elements (kpm_weighted.cuh), one state per thread; the
-// elements and their order are those of spin_step_kernel.
+// elements and their order are those of spin_step_kernel; in fixed point they are
+// made of whole numbers, rounded once, to 2^-59.
 struct SpinListArgs {
   uint4 *lists;
   SpinTablesDev tb;
   int stride;
   uint32_t crow, zero_chunk;
+  const FxScaled *couplings;  // fixed point: [n_sectors][n_bonds] J/a, and
+  const int64_t *c0;          // [n_sectors] 2/a (s^2 sum J - b), in 2^-59
   int *flag;
 };
 
@@ -448,29 +471,48 @@ __global__ void __launch_bounds__(32)
       const uint64_t code =
           sd.Q < 0 ? spin_full_code(rank, a.tb) : spin_unrank((uint32_t)rank, sd.Q, tile.b_last, hb, a.tb);
       uint4 *L = a.lists + (size_t)row * a.stride;
-      double sum = 0.0;
       uint32_t e = 1;
-      auto element = [&](double c) {
-        if (FIXED) {
-          const FxCoef k = fx_coef_device(c, out_of_range);
-          return make_uint2((unsigned)k.h, k.l);
+      uint2 k;
+      if (FIXED) {
+        int64_t sum = 0;  // of |coefficients|, in units of 2^-51
+        auto coefficient = [&](i128 c) {
+          const bool out = c > kFxCoefUnits || -c > kFxCoefUnits;
+          out_of_range |= out;
+          if (!out) sum += llabs((int64_t)c) >> 8;
+          const FxCoef f = fx_limbs_of(out ? 0 : (int64_t)c);
+          return make_uint2((unsigned)f.h, f.l);
+        };
+        const FxScaled *fx = a.couplings + (size_t)tile.sector * bd.n_bonds;
+        spin_neighbours(code, rank, sd, a.tb, bd, [&](int64_t nrow, int b, int q, int p) {
+          const FxScaled f = fx[b];
+          const uint2 v = coefficient(((i128)f.F * bd.ladder[8 * q + p] + ((i128)1 << (f.e - 2))) >> (f.e - 1));
+          L[e++] = make_uint4((uint32_t)nrow * a.crow, v.x, v.y, 0);
+        });
+        i128 d = 0;  // J/(2a) ((2 m_i)(2 m_j) - (2s)^2) over the bonds, in units of 2^-75
+        for (int b = 0; b < bd.n_bonds; ++b) {
+          const int mm = (2 * digit(code, bd.bi[b]) - a.tb.two_s) * (2 * digit(code, bd.bj[b]) - a.tb.two_s) -
+                         a.tb.two_s * a.tb.two_s;
+          const FxScaled f = fx[b];
+          const int sh = f.e - 74;
+          d += sh <= 0 ? ((i128)f.F * mm) << -sh : ((i128)f.F * mm + ((i128)1 << (sh - 1))) >> sh;
         }
-        const float hi = (float)c;
-        return make_uint2(__float_as_uint(hi), __float_as_uint((float)(c - (double)hi)));
-      };
-      const double diag = spin_apply(code, rank, sd, a.tb, bd, [&](int64_t nrow, double amp) {
-        const double c = A * amp;
-        sum += fabs(c);
-        const uint2 k = element(c);
-        L[e++] = make_uint4((uint32_t)nrow * a.crow, k.x, k.y, 0);
-      });
+        k = coefficient(((d + (1 << 15)) >> 16) + a.c0[tile.sector]);
+        out_of_range |= sum > kFxRowUnits;
+      } else {
+        auto element = [](double c) {
+          const float hi = (float)c;
+          return make_uint2(__float_as_uint(hi), __float_as_uint((float)(c - (double)hi)));
+        };
+        const double diag = spin_apply(code, rank, sd, a.tb, bd, [&](int64_t nrow, double amp) {
+          const uint2 v = element(A * amp);
+          L[e++] = make_uint4((uint32_t)nrow * a.crow, v.x, v.y, 0);
+        });
+        k = element(A * (diag - sd.b));
+      }
       const uint32_t cnt = e - 1;
       while ((e - 1) % kWeightedBatch != 0) L[e++] = make_uint4(a.zero_chunk, 0, 0, 0);
       int q = 0;
       for (int i = 0; i < a.tb.N; ++i) q += digit(code, i);
-      const double c = A * (diag - sd.b);
-      if (FIXED) out_of_range |= !(sum + fabs(c) <= kFxMaxRow);
-      const uint2 k = element(c);
       L[0] = make_uint4(cnt, k.x, k.y, (unsigned)(2 * q - a.tb.N * a.tb.two_s));
     }
   }
@@ -640,10 +682,45 @@ struct SpinRun {
   WeightedRun wr;
   size_t list_bytes() const {
     return weighted ? align256((size_t)plan.total_rows * wr.stride * sizeof(uint4)) +
-                          align256((size_t)plan.n_sectors * sizeof(double))
+                          align256((size_t)plan.n_sectors * sizeof(double)) +
+                          align256((size_t)plan.n_sectors * bonds.n_bonds * sizeof(FxScaled)) +
+                          align256((size_t)plan.n_sectors * sizeof(int64_t))
                     : 0;
   }
 };
+
+// Couplings J/a of every sector and bond, and the rest of the diagonal; false when one
+// is out of the fixed-point range.
+bool fixed_spin_couplings(const kpm_spin_model *m, const SpinPlan &p, const double *a, const double *b,
+                          std::vector<FxScaled> *couplings, std::vector<int64_t> *c0) {
+  couplings->assign((size_t)p.n_sectors * m->n_bonds, FxScaled{0, 62, 0});
+  c0->assign(p.n_sectors, 0);
+  const double s = 0.5 * m->two_s;
+  // s^2 sum_b J_b, the energy of the largest total spin: a level of every sector, so
+  // that its distance from b is within the range where the diagonal is
+  FxPair top{0.0, 0.0};
+  for (int k = 0; k < m->n_bonds; ++k) top = fx_pair_add(top, 0.25 * m->J[k]);
+  top = fx_pair_mul(top, FxPair{(double)m->two_s * m->two_s, 0.0});
+  for (int i = 0; i < p.n_sectors; ++i) {
+    const FxPair A = fx_two_over(a[i]);
+    FxPair d = fx_pair_mul(A, fx_pair_add(top, -b[i]));
+    if (p.dim[i] == 1) {
+      // one state: no couplings, and b is this sum in FP64 while a may be tiny
+      double diag = 0.0;
+      for (int k = 0; k < m->n_bonds; ++k) diag += m->J[k] * s * s;
+      d = FxPair{2.0 * (1.0 / a[i]) * (diag - b[i]), 0.0};
+    } else {
+      for (int k = 0; k < m->n_bonds; ++k) {
+        const FxPair c = fx_pair_mul(A, FxPair{0.5 * m->J[k], 0.0});
+        if (!(std::fabs(c.h) <= kFxMaxCoef)) return false;
+        (*couplings)[(size_t)i * m->n_bonds + k] = fx_scaled(c);
+      }
+    }
+    if (!(std::fabs(d.h) <= kFxMaxCoef)) return false;
+    (*c0)[i] = fx_units(d);
+  }
+  return true;
+}
 
 int64_t spin_tile_states(const RowLayout &lay, int64_t rows) {
   const int64_t big = (int64_t)16 * kWarps * lay.gpw;
@@ -881,6 +958,20 @@ int spin_moments_run(const kpm_spin_model *model, int32_t n_sectors, const int32
     la.crow = (uint32_t)(r.lay.Rp / r.lay.vec_width);
     la.zero_chunk = (uint32_t)r.plan.total_rows * la.crow;
     la.flag = flag;
+    la.couplings = nullptr;
+    la.c0 = nullptr;
+    if (r.fixed) {
+      std::vector<FxScaled> couplings;
+      std::vector<int64_t> c0;
+      if (!fixed_spin_couplings(model, r.plan, a, b, &couplings, &c0)) {
+        *flags = kFlagRange;
+        return KPM_OK;
+      }
+      PackedUpload up(ar, s);
+      KPM_TRY(up.add(couplings, &la.couplings));
+      KPM_TRY(up.add(c0, &la.c0));
+      KPM_TRY(up.send());
+    }
     const int lgrid = (int)std::min<int64_t>((int64_t)r.plan.tiles.size(), (int64_t)32 * sm_count());
     if (r.fixed)
       spin_build_lists_kernel<true><<<lgrid, 32, 0, s>>>(la, r.bonds);

@@ -290,3 +290,91 @@ def test_weighted_sums_have_no_bias(n, count, R):
     for q in ("mu", "mu_M", "mu_M2"):
         assert np.abs(got[0][q][0, 1::2] + got[1][q][0, 1::2]).max() <= 4.5e-16, q
         assert np.abs(got[0][q][0, 0::2] - got[1][q][0, 0::2]).max() <= 4.5e-16, q
+
+
+# ---------------------------------------------------------------- coefficients
+# Against the recursion in extended precision with the same a and b (80 or 128 bits).  A level
+# of H' that is off by d moves mu_n by up to n d.  Coefficients are rounded to 2^-60: with 8
+# (spin 5/2: 4) bonds d <= 9 2^-60 (diagonal and flips: twice), at n = 1000 so 1.6e-14; the
+# vectors' roundings of 0.29/U in the mean square add 4 sqrt(n sum U_k^2) 0.29/(U sqrt(DR)),
+# below 4e-15 at D R = 768 for a mean square of 10 of the U_k, five sigma; sums 1e-15.
+def _extended(codes, diag, rows, cols, vals, a, b, K, R, seed, M):
+    L = np.longdouble
+    mask = (1 << 64) - 1
+
+    def sm(x):
+        z = (x + 0x9E3779B97F4A7C15) & mask
+        z = ((z ^ (z >> 30)) * 0xBF58476D1CE4E5B9) & mask
+        z = ((z ^ (z >> 27)) * 0x94D049BB133111EB) & mask
+        return z ^ (z >> 31)
+
+    h = [sm(sm(seed) ^ r) for r in range(R)]
+    x = np.array([[-1 if sm(hr ^ int(c)) >> 63 else 1 for hr in h] for c in codes]).astype(L)
+    a, b = L(a), L(b)
+    order = np.argsort(rows, kind="stable")
+    rows, cols, vals = rows[order], cols[order], vals[order][:, None]
+    starts = np.searchsorted(rows, np.arange(len(codes)))
+    has = np.bincount(rows, minlength=len(codes)) > 0
+
+    def hp(v):
+        off = np.zeros_like(v)
+        off[has] = np.add.reduceat(vals * v[cols], starts[has], axis=0)
+        return ((diag[:, None] - b) * v + off) / a
+
+    def dots(y):
+        return [np.array([(w * (u * y).sum(1)).sum() for w in (1, M, M * M)]) / (L(len(codes)) * R) for u in (x,)][0]
+
+    y = hp(x)
+    d = [dots(x), None]
+    d[1] = dots(y)
+    f0, f1 = d
+    for _ in range(1, K // 2):
+        x, y = y, 2 * hp(y) - x
+        d += [2 * dots(x) - f0, 2 * dots(y) - f1]
+    return np.array(d).T
+
+
+def test_coefficients_small_sectors():
+    n, J, a, b, K, R = 8, 1.0073, 3.0917, -0.8931, 2000, 3
+    L = np.longdouble
+    codes = np.arange(1 << n)
+    diag, rows, cols = np.zeros(1 << n, L), [], []
+    for i in range(n):
+        m = (1 << i) | (1 << (i + 1) % n)
+        anti = ((codes & m) != 0) & ((codes & m) != m)
+        diag += L(J) * np.where(anti, L(-0.25), L(0.25))
+        rows.append(codes[anti])
+        cols.append(codes[anti] ^ m)
+    rows, cols = np.concatenate(rows), np.concatenate(cols)
+    M = np.array([bin(c).count("1") - n / 2 for c in codes]).astype(L)
+    ref = _extended(codes, diag, rows, cols, np.full(len(rows), L(J) / 2), a, b, K, R, 5, M)
+    got = kpm.moments(W.ring(n, J), [-1], K, R, 5, a=[a], b=[b])
+    for i, q in enumerate(("mu", "mu_M", "mu_M2")):
+        assert np.abs(got[q][0] - ref[i]).max() <= 2.2e-14 * (1, 1.5, n / 4)[i], q
+
+
+def test_coefficients_spin():
+    n, two_s, J, a, b, K, R = 4, 5, 1.0073, 28.1237, -2.4931, 2000, 1
+    L = np.longdouble
+    d = two_s + 1
+    rank = np.arange(d ** n)
+    q = np.stack([(rank // d ** i) % d for i in range(n)])
+    codes = sum(q[i].astype(np.int64) << (3 * i) for i in range(n))
+    where = {int(c): k for k, c in enumerate(codes)}
+    m2 = 2 * q - two_s
+    diag, rows, cols, vals = np.zeros(len(rank), L), [], [], []
+    for i in range(n):
+        j = (i + 1) % n
+        diag += L(J) / 4 * (m2[i] * m2[j])
+        for s in (1, -1):
+            p, r = (i, j) if s == 1 else (j, i)
+            k = (two_s - q[p]) * (q[p] + 1) * q[r] * (two_s - q[r] + 1)
+            ok = k > 0
+            rows.append(rank[ok])
+            cols.append(np.array([where[int(c)] for c in codes[ok] + (1 << 3 * p) - (1 << 3 * r)]))
+            vals.append(L(J) / 2 * np.sqrt(k[ok].astype(L)))
+    ref = _extended(codes, diag, np.concatenate(rows), np.concatenate(cols), np.concatenate(vals), a, b, K, R,
+                    5, m2.sum(0).astype(L) / 2)
+    got = kpm.spin_moments(W.ring(n, J), two_s, [-1], K, R, 5, [a], [b])
+    for i, (k, scale) in enumerate((("mu", 1), ("mu_M", 3.5), ("mu_M2", 12))):
+        assert np.abs(got[k][0] - ref[i]).max() <= 2.2e-14 * scale, k
