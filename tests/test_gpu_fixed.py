@@ -378,3 +378,14 @@ def test_coefficients_spin():
     got = kpm.spin_moments(W.ring(n, J), two_s, [-1], K, R, 5, [a], [b])
     for i, (k, scale) in enumerate((("mu", 1), ("mu_M", 3.5), ("mu_M2", 12))):
         assert np.abs(got[k][0] - ref[i]).max() <= 2.2e-14 * scale, k
+
+
+# ---------------------------------------------------------------- dot products of FP32 spin runs
+# They are sums of exact products as if in FP64.  All components of v_0 are +-x, so mu_0 is
+# D x^2; tolerance: 30 roundings of FP64 (the sum over a tile's lanes, the tiles and the vectors).
+@pytest.mark.parametrize("two_s,n,Q,R", [(2, 12, 12, 100), (5, 8, 20, 60), (5, 5, 12, 4)])
+def test_dot_products_of_fp32_spin_runs(two_s, n, Q, R):
+    D = kpm.lib().kpm_spin_sector_dim(n, two_s, Q)
+    got = kpm.spin_moments(W.ring(n), two_s, [Q], 2, R, 5, [90.0], [0.0], precision="fp32")
+    x = float(np.float32(1.0 / np.sqrt(float(D))))
+    assert abs(got["mu"][0, 0] - D * x * x) <= 30 * 2.0 ** -53
