@@ -1342,8 +1342,15 @@ int prepare_run(const kpm_model *m, int n_sectors, const int32_t *n_up, int K, i
       run->lay.gpw = 32 / run->lay.G;
       if (list_smem_bytes(run->lay.gpw, stride_of(fixed_batch(2))) > kMaxListSmem) run->lay = single;
     }
-    const int stride = stride_of(run->fixed ? fixed_batch(run->lay.cpl)
-                                            : list_pad(precision, run->lay.cpl, run->lay.gpw));
+    int stride = stride_of(run->fixed ? fixed_batch(run->lay.cpl)
+                                      : list_pad(precision, run->lay.cpl, run->lay.gpw));
+    if (run->fixed && list_smem_bytes(run->lay.gpw, stride) > kMaxListSmem) {
+      // rows of few chunks (16 states per warp): the padded lists do not fit, the FP64
+      // kernel's, which are not padded, may (J1-J2 chain N = 18, R = 4, K = 200: 2.9 ms, with the
+      // matrix-free kernel 6.8 ms)
+      run->fixed = false;
+      stride = stride_of(list_pad(precision, run->lay.cpl, run->lay.gpw));
+    }
     if (list_smem_bytes(run->lay.gpw, stride) <= kMaxListSmem)
       run->list_stride = stride;
     else

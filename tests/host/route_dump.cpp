@@ -20,8 +20,12 @@ int main() {
     kpm_model m{N, nb, bi.data(), bj.data(), J.data()};
     kpm::MomentsRun r;
     const int rc = kpm::prepare_run(&m, ns, up.data(), K, R, precision, &r);
-    std::printf("%d small %d fixed %d weighted %d stride %d unit %lld\n", rc, r.small, r.fixed,
-                r.weighted, r.list_stride, (long long)r.fx_unit);
+    kpm::Knobs fp64;  // the same without fixed point
+    fp64.fixed = 0;
+    kpm::MomentsRun p;
+    if (kpm::prepare_run(&m, ns, up.data(), K, R, precision, &p, fp64) != rc) return 1;
+    std::printf("%d small %d fixed %d weighted %d stride %d unit %lld fp64_stride %d\n", rc, r.small,
+                r.fixed, r.weighted, r.list_stride, (long long)r.fx_unit, p.list_stride);
   }
   return 0;
 }

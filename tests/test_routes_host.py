@@ -56,3 +56,13 @@ def test_fixed_point_rounds_no_more_than_fp64(route, n, k):
                 assert 0.29 / r["unit"] <= 2 ** -54.05, (kind, count, r)
                 seen.add(kind)
     assert seen == {"one", "two", "own"}
+
+
+# Lists padded for the fixed-point kernel may not fit where those of the FP64 kernel do: a run
+# that had lists keeps them, for every number of vectors.
+@pytest.mark.parametrize("model", [W.ring(18), W.j1j2_chain(18, 1.0, 0.4), W.ladder(18), W.sawtooth(18, -1.0, 0.4),
+                                   W.j1j2_square(4, 5, 1.0, 0.5)], ids=lambda m: m.name)
+def test_fixed_point_keeps_the_lists(route, model):
+    for R in list(range(3, 34)) + [48, 64, 65, 100, 128, 129]:
+        r = route(model, [model.n_sites // 2], R)
+        assert r["stride"] > 0 or r["fp64_stride"] == 0, (R, r)
