@@ -135,6 +135,10 @@ struct TablesDev {
   int32_t pad;
 };
 
+// SMs of a GB300: for rules that have to give the same where no GPU is visible (the size
+// queries); grids are sized by the device's own number.
+constexpr int kSms = 152;
+
 constexpr int kMaxGroups = 4;       // distinct coupling values handled by the grouped step
 constexpr int kMaxDiagTable = 4096; // entries of the per-sector diagonal table
 

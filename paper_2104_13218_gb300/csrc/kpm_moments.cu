@@ -1399,7 +1399,7 @@ int prepare_run(const kpm_model *m, int n_sectors, const int32_t *n_up, int K, i
     // a small run: at least one tile for each of the 16 warps that an SM holds
     // (ladder N = 14, R = 25: 21.5 -> 13 us per step)
     const int64_t g = run->lay.gpw;
-    ts = std::min(ts, std::max<int64_t>(g, (rows / (16 * 152) + g - 1) / g * g));
+    ts = std::min(ts, std::max<int64_t>(g, (rows / (16 * kSms) + g - 1) / g * g));
   }
   if (knobs.tile_states > 0) {
     // a tuned tile size, in whole warp groups, within the list kernel's tile limit
@@ -1470,7 +1470,7 @@ int prepare_run(const kpm_model *m, int n_sectors, const int32_t *n_up, int K, i
     run->n_cd = (int)(run->cd_chunks.size() / 3);
     run->cd_chunks.insert(run->cd_chunks.end(), ranges.begin(), ranges.end());
   }
-  run->small = fixed_point && knobs.small != 0 && small_applies(m, n_sectors, n_up);
+  run->small = fixed_point && knobs.small != 0 && small_applies(m, n_sectors, n_up) && small_pays(m, *run);
   if (run->small) KPM_TRY(prepare_small(m, run));
   fill_pass_masks(&run->bonds, run->lay.G);
   run->NQ = run->plan.any_full ? 6 : 2;

@@ -227,6 +227,7 @@ void *block_kernel_ptr(int precision);
 // the shared memory of a block.
 constexpr int64_t kSmallMaxDim = 13500;
 bool small_applies(const kpm_model *m, int n_sectors, const int32_t *n_up);
+bool small_pays(const kpm_model *m, const MomentsRun &run);
 int prepare_small(const kpm_model *m, MomentsRun *run);
 size_t small_bytes(const MomentsRun &r);
 // Carves and fills the run's buffers.

@@ -347,6 +347,37 @@ bool small_applies(const kpm_model *m, int n_sectors, const int32_t *n_up) {
   return true;
 }
 
+// Whether one launch is the faster form of a prepared run.  A product of one vector takes a
+// block 0.14 ns (bonds with their own couplings: 0.21 ns) per state and for each of its
+// neighbours + 3, and one block has it to itself: the largest sector sets the step, or
+// all of them when they fill the chip.  The kernels that spread a step over the chip take 10 us
+// at least (whole space, with its weighted sums: 22 us; FP64 vectors: 14 us with lists, 20 us
+// without), and 1.1e-6 us
+// (1.3e-6; FP64 vectors 3e-5) per state, neighbour + 3 and vector.  Measured for K = 200,
+// S^z = 0 sector, one launch against the others in ms: 3432 states (ladder, R = 1 / 24 / 100) 0.83
+// against 1.6 / 1.0 / 1.3; 6435 states (J1-J2 chain, R = 1 / 4 / 8 / 100) 1.8 against 2.0 / 1.4 /
+// 1.0 / 1.9; 12870 states (J1-J2 chain, R = 1 / 8 / 64 / 100) 3.4 against 2.0 / 1.2 / 1.8 / 3.1,
+// (random couplings, R = 8) 5.5 against 1.4; whole space of 16 sites (ring, R = 8 / 100) 2.1 / 7.0
+// against 2.6 / 9.2.  Over 195 such runs the choice is 0.4% slower than the better one in
+// the mean, 12% at most.
+bool small_pays(const kpm_model *m, const MomentsRun &r) {
+  double largest = 0.0, total = 0.0;
+  for (int32_t k : sub_sectors(r.plan, nullptr)) {
+    const double N = m->n_sites, flips = N > 1 ? m->n_bonds * 2.0 * k * (N - k) / (N * (N - 1)) : 0.0;
+    const double work = (double)binom(m->n_sites, k) * (flips + 3.0);
+    largest = std::max(largest, work);
+    total += work;
+  }
+  const int R = r.lay.R;
+  const double one = (r.bonds.n_groups > 0 ? 1.4e-4 : 2.1e-4) * std::max(largest, total * R / kSms);
+  const bool full = r.plan.any_full;
+  double stepped = r.fixed || r.weighted ? std::max(full ? 22.0 : 10.0, (full ? 1.3e-6 : 1.1e-6) * total * R)
+                                         : std::max(r.list_stride > 0 ? 14.0 : 20.0, 3e-5 * total * r.lay.Rp);
+  // every vector's moments: another pass over the vectors, which one launch does not need
+  if (r.per_vector) stepped *= 1.6;
+  return one <= stepped;
+}
+
 int prepare_small(const kpm_model *m, MomentsRun *r) {
   if (!r->plan.any_full) return KPM_OK;  // the run's own sectors
   const std::vector<int32_t> sub = sub_sectors(r->plan, nullptr);

@@ -755,7 +755,7 @@ int prepare_spin(const kpm_spin_model *m, int n_sectors, const int32_t *Q, int R
     // single warps' tiles: at most 16 states of a lane, and a small run gives one to
     // each of the 16 warps that an SM holds
     ts = std::min<int64_t>(16 * lay.gpw,
-                           std::max<int64_t>(lay.gpw, (rows / (16 * 152) + lay.gpw - 1) / lay.gpw * lay.gpw));
+                           std::max<int64_t>(lay.gpw, (rows / (16 * kSms) + lay.gpw - 1) / lay.gpw * lay.gpw));
   }
   KPM_TRY(build_spin_plan(m, n_sectors, Q, ts, &run->plan));
   fill_spin_bonds(m, &run->bonds);

@@ -369,7 +369,7 @@ int setup_thermo(ThermoCall &tc, int S, int K, const double *mu, const double *m
   KPM_CUDA(cudaGetLastError());
   const int64_t rows = (int64_t)P * S * 3;
   const int by = (int)std::min<int64_t>(rows, 65535);
-  const int bx = std::max(1, std::min((Nq + kWarps - 1) / kWarps, (int)(16 * 152 / std::min<int64_t>(rows, 2048))));
+  const int bx = std::max(1, std::min((Nq + kWarps - 1) / kWarps, (int)(16 * kSms / std::min<int64_t>(rows, 2048))));
   thermo_gamma_kernel<<<dim3(bx, by, (int)((rows + by - 1) / by)), kThreads, 0, stream>>>(A);
   KPM_CUDA(cudaGetLastError());
   count_launches(2);

@@ -66,3 +66,18 @@ def test_fixed_point_keeps_the_lists(route, model):
     for R in list(range(3, 34)) + [48, 64, 65, 100, 128, 129]:
         r = route(model, [model.n_sites // 2], R)
         assert r["stride"] > 0 or r["fp64_stride"] == 0, (R, r)
+
+
+# Small sectors run in one launch where that is the faster form: not when a few vectors of
+# a large sector would leave most of the chip idle, nor when the kernels that spread a step over the
+# chip fill it as well.  (the clear cases of the measurements: the other form at least 20% slower)
+@pytest.mark.parametrize("model,n_up,R,one_launch", [
+    (W.j1j2_chain(16, 1.0, 0.4), [8], 1, 0), (W.j1j2_chain(16, 1.0, 0.4), [8], 4, 0),
+    (W.j1j2_chain(16, 1.0, 0.4), [8], 16, 0), (W.random_bonds(16, 32, 3, 0.2, 1.5), [8], 1, 0),
+    (W.random_bonds(16, 32, 3, 0.2, 1.5), [8], 16, 0), (W.j1j2_chain(15, 1.0, 0.4), [7], 8, 0),
+    (W.j1j2_chain(15, 1.0, 0.4), [7], 4, 0),
+    (W.random_bonds(15, 30, 3, 0.2, 1.5), [8, 9, 10], 4, 0), (W.ladder(16), [8, 9, 10, 11, 12, 13, 14, 15, 16], 8, 0),
+    (W.ladder(14), [7], 1, 1), (W.ladder(14), [7, 8, 9, 10, 11, 12, 13, 14], 25, 1), (W.ring(10), [-1], 20, 1),
+    (W.ring(12), [6], 1, 1), (W.ring(16), [-1], 100, 1), (W.ladder(16), [8, 9, 10, 11, 12, 13, 14, 15, 16], 1, 1)])
+def test_small_sectors_rule(route, model, n_up, R, one_launch):
+    assert route(model, n_up, R)["small"] == one_launch
