@@ -1985,13 +1985,6 @@ int launch_assemble(const MomentsRun &r, double *mu, double *mu_M, double *mu_M2
   return KPM_OK;
 }
 
-bool scratch_fits(size_t need, const void *workspace, size_t ws_bytes) {
-  if (workspace != nullptr) return need <= ws_bytes;
-  if (need < ((size_t)1 << 30)) return true;  // the allocation itself will tell
-  size_t free_b = 0, total_b = 0;
-  return cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || need <= free_b;
-}
-
 int prepare_job(const kpm_model *m, int n_sectors, const int32_t *n_up, int K, int R,
                 int precision, MomentsJob *job, const Knobs &knobs, int vectors,
                 bool per_vector) {
@@ -2207,14 +2200,19 @@ int moments_impl(const kpm_model *model, int32_t n_sectors, const int32_t *n_up,
   const size_t out_bytes = align256(SK * sizeof(double));
   const size_t r_bytes = mu_r ? align256(SK * R * sizeof(double)) : 0;
   const size_t out_need = on_device ? 0 : 3 * out_bytes + r_bytes;
-  if (!scratch_fits(job_bytes(job) + out_need, workspace, ws_bytes)) {
-    job = MomentsJob();
-    KPM_TRY(prepare_job(model, n_sectors, n_up, n_moments, R, o.precision, &job, least_scratch(knobs),
-                        o.vectors, o.per_vector != 0));
-  }
-  const size_t need = job_bytes(job) + out_need;
   Workspace ws;
-  KPM_TRY(ws.acquire(workspace, ws_bytes, need, stream));
+  int rc = ws.acquire(workspace, ws_bytes, job_bytes(job) + out_need, stream);
+  if (rc == KPM_ENOMEM) {
+    MomentsJob least;
+    KPM_TRY(prepare_job(model, n_sectors, n_up, n_moments, R, o.precision, &least, least_scratch(knobs),
+                        o.vectors, o.per_vector != 0));
+    if (job_bytes(least) < job_bytes(job)) {
+      job = std::move(least);
+      clear_error();
+      rc = ws.acquire(workspace, ws_bytes, job_bytes(job) + out_need, stream);
+    }
+  }
+  KPM_TRY(rc);
   Arena arena{reinterpret_cast<char *>(ws.ptr), ws.size, 0};
   double *dmu = mu, *dmuM = mu_M, *dmuM2 = mu_M2, *dmur = mu_r;
   if (!on_device) {

@@ -25,14 +25,14 @@ struct Knobs {
 };
 
 // The knobs that need the least scratch (no lists with matrix elements, no
-// padded lists): for calls whose memory does not hold the default run.
+// padded lists): for calls whose memory does not hold the default run, that is
+// whose workspace is too small or whose allocation fails.
 inline Knobs least_scratch(Knobs k) {
   k.weighted = 0;
   k.fixed = 0;
   k.small = 0;
   return k;
 }
-bool scratch_fits(size_t need, const void *workspace, size_t ws_bytes);
 
 // Coefficients of H' per sector and kind of step (first: A = 1/a, later:
 // A = 2/a), computed on the host once per run: the diagonal A (d - b) for every

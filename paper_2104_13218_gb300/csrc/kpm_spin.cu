@@ -902,17 +902,15 @@ int spin_moments_run(const kpm_spin_model *model, int32_t n_sectors, const int32
                        align256(2 * r.plan.tiles.size() * r.NQ * 8) +
                        align256((size_t)S * n_sectors * r.NQ * 8) + align256((size_t)S * 4) + 256 +
                        (on_device ? 0 : 3 * align256(SK * 8)) + 4096;
-  if (r.weighted && bytes > ((size_t)1 << 30)) {
-    size_t free_b = 0, total_b = 0;
-    KPM_CUDA(cudaMemGetInfo(&free_b, &total_b));
-    if (bytes > free_b) {
-      *flags = kFlagRange;
-      return KPM_OK;
-    }
-  }
   StreamAlloc mem;
   mem.s = s;
-  KPM_TRY(scratch_alloc(&mem.p, bytes, s));
+  const int rc = scratch_alloc(&mem.p, bytes, s);
+  if (rc == KPM_ENOMEM && r.weighted) {
+    clear_error();
+    *flags = kFlagRange;
+    return KPM_OK;
+  }
+  KPM_TRY(rc);
   Arena ar{reinterpret_cast<char *>(mem.p), bytes, 0};
   char *vA = ar.take<char>(r.vec_bytes), *vB = ar.take<char>(r.vec_bytes);
   const size_t slot = r.plan.tiles.size() * r.NQ;
