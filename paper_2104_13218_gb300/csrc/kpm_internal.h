@@ -251,6 +251,8 @@ struct Workspace {
   bool idle = false;  // the stream was synchronised after the last use
   cudaStream_t stream = nullptr;
   int acquire(void *user, size_t user_bytes, size_t need, cudaStream_t s);
+  // Makes room for `need` bytes (the contents are lost); KPM_ENOMEM for a caller's region.
+  int grow(size_t need);
   ~Workspace();
 };
 

@@ -330,6 +330,15 @@ int Workspace::acquire(void *user, size_t user_bytes, size_t need, cudaStream_t 
   return KPM_OK;
 }
 
+int Workspace::grow(size_t need) {
+  if (need <= size) return KPM_OK;
+  KPM_REQUIRE(owned, KPM_ENOMEM, "workspace of %zu bytes, need %zu", size, need);
+  scratch_free(ptr, stream);
+  ptr = nullptr;
+  size = 0;
+  return acquire(nullptr, 0, need, stream);
+}
+
 Workspace::~Workspace() {
   if (owned && ptr) {
     scratch_free(ptr, stream);

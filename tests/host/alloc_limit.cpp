@@ -97,5 +97,26 @@ int main() {
       return kpm_spin_moments(&sm, 1, &Q, &a, &b, 20, 20, 5, 0, precision, mu.data(), nullptr, nullptr, 0, nullptr);
     });
   }
+  // The gradient's fixed-point sweep needs four vectors; the checkpoints of the FP64 sweep
+  // (K = 200: eight more) are not to be asked for.
+  {
+    const int n = 14, K = 200, R = 20;
+    const Model m(n, false);
+    const kpm_model km = m.of(n);
+    const int32_t up = n / 2;
+    std::vector<int32_t> cls(km.n_bonds);
+    for (int b = 0; b < km.n_bonds; ++b) cls[b] = b / n;
+    std::vector<double> g(K);
+    for (int k = 0; k < K; ++k) g[k] = std::cos(1.0 + k);
+    const size_t vec = (size_t)kpm_sector_dim(n, up) * R * 8;
+    for (double a : {30.0, 1.0}) {  // (the second leaves the range: the FP64 sweep needs them)
+      const double b = 0.0;
+      check(a > 1.0 ? "gradient-inside" : "gradient-outside", [&](std::vector<double> &d) {
+        d.assign(2, NAN);
+        return kpm_moments_backward(&km, cls.data(), 2, 1, &up, &a, &b, K, R, 5, 0, KPM_FP64, 0, g.data(), nullptr,
+                                    nullptr, d.data(), 0, nullptr, 0, nullptr);
+      }, 7 * vec);
+    }
+  }
   return 0;
 }

@@ -36,6 +36,9 @@ def test_failed_allocations(tmp_path):
         name, rc, rc_limit, diff = line.split()[:4]
         tol = 1e-5 if name in ("moments-0-12-1", "moments-0-16-1") else 1e-10
         # (grouped FP32 runs have no form with less scratch)
+        if name == "gradient-outside":
+            assert int(rc) == 0 and int(rc_limit) == 2, line
+            continue
         if name == "moments-0-16-1":
             assert int(rc) == 0 and int(rc_limit) in (0, 2), line
             continue
@@ -67,3 +70,22 @@ def test_moments_in_a_small_workspace(R, precision):
                 assert ((got[q] - ref[q]).abs() / scale).max() <= (1e-10 if precision == "fp64" else 1e-5), (q, mid)
         if model.n_bonds == 37 and (R > 4 or precision == "fp64"):  # (FP32 rows of one lane have no lists)
             assert hi < 0.8 * size  # without the lists with matrix elements
+
+
+# A caller's workspace without room for the FP64 sweep's checkpoints: enough for a run in fixed
+# point, KPM_ENOMEM for one that leaves the range; the queried size serves both.
+def test_gradient_in_a_small_workspace():
+    model, n_up, K, R = W.j1j2_chain(14, 1.0, 0.4), [7], 200, 20
+    cls = model.classes()
+    g = {"mu": np.cos(1.0 + np.arange(K))[None]}
+    size = kpm.moments_backward_workspace_size(model, n_up, K, R)
+    small = size - 2 * 4 * 3432 * R * 8  # the pairs of every 32nd of 100 steps
+    for bytes_, a, enough in ((small, 30.0, True), (small, 1.0, False), (size, 1.0, True)):
+        args = (model, cls, 2, n_up, [a], [0.0], K, R, 5, g)
+        ws = torch.full((bytes_ + 4096,), 0xFF, dtype=torch.uint8, device="cuda")
+        if not enough:
+            with pytest.raises(kpm.KPMError, match="KPM_ENOMEM"):
+                kpm.moments_backward(*args, workspace=ws)
+            continue
+        got, ref = kpm.moments_backward(*args, workspace=ws), kpm.moments_backward(*args)
+        assert np.array_equal(got, ref), (a, got, ref)
