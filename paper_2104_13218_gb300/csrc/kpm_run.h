@@ -64,10 +64,6 @@ struct BlockBondsDev {
 constexpr int kVecRademacher = 0;
 constexpr int kVecBasis = 1;
 
-// Bits of a run's device flag.
-constexpr int kFlagBounds = 1;  // some |mu_n| > 1 + 1e-6
-constexpr int kFlagRange = 2;   // a component left the fixed-point range
-
 // Device state of a small-sector run (kpm_small.cu).
 struct FxCoef;
 struct SmallRun {

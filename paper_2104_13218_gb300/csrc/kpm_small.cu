@@ -248,7 +248,13 @@ __global__ void __launch_bounds__(kSmallThreads, 1) small_run_kernel(const __gri
       const i128 v = warp_sums<2>(acc);
       if ((lane & 15) == 0) slot[(lane >> 4) * 32 + warp] = v;
     }
-    __syncthreads();
+    // a run that left the range ends (its results are not used): looked at every 16 steps
+    if ((n & 15) == 0) {
+      const bool out = top >= 2 * a.lim_hi || (threadIdx.x == 0 && (__ldcg(a.flag) & kFlagRange));
+      if (__syncthreads_or(out)) break;
+    } else {
+      __syncthreads();
+    }
     // one warp (another at every step) adds the warps' sums while the others go on;
     // this slot is written again only after the next barrier
     if (warp == n % nw) {

@@ -5,6 +5,8 @@ Tolerance of moments within the spectral interval: 1e-12, a hundred times below 
 tolerance of the parity tests.  A component is rounded to U/sqrt(D) 2^-1 with
 U >= 2^49 (255 bonds), so a step adds at most 2^-50 of the vector's norm, and
 n steps at most n^2 2^-50 to mu_n: 2e-13 at n = 15 matrix-vector products."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -389,3 +391,28 @@ def test_dot_products_of_fp32_spin_runs(two_s, n, Q, R):
     got = kpm.spin_moments(W.ring(n), two_s, [Q], 2, R, 5, [90.0], [0.0], precision="fp32")
     x = float(np.float32(1.0 / np.sqrt(float(D))))
     assert abs(got["mu"][0, 0] - D * x * x) <= 30 * 2.0 ** -53
+
+
+def _step_launches(call):
+    """Device time (ms) and number of the step launches that a call makes."""
+    ms, n = ctypes.c_double(), ctypes.c_int64()
+    kpm.lib().kpm_profile_enable(1)
+    call()
+    kpm.lib().kpm_profile_read(ctypes.byref(ms), ctypes.byref(n), None)
+    kpm.lib().kpm_profile_enable(0)
+    return ms.value, n.value
+
+
+# A run that leaves the range in its first ten steps or so (levels of H' down to -1.6) does not pay for the others: its step launches
+# take no longer than those of the FP64 run that replaces it (unit vectors are run in FP64) and a
+# part of a fixed-point run's.
+def test_abandoned_run_stops():
+    def step_ms(a, **kw):
+        for _ in range(2):
+            r = _step_launches(lambda: kpm.moments(W.ring(20), [10], 200, 20, 5, a=[a], b=[-1.0],
+                                                   allow_ebounds=True, device=True, **kw))
+        return r
+
+    fixed, fp64, left = step_ms(30.0), step_ms(30.0, vectors="basis"), step_ms(5.0)
+    assert left[1] == fixed[1] + fp64[1] and fp64[0] > 2 * fixed[0]
+    assert left[0] < fp64[0] + 0.5 * fixed[0], (fixed, fp64, left)
