@@ -286,7 +286,8 @@ struct BoundsLayout {
 constexpr size_t kBoundsListMaxBytes = (size_t)2 << 30;
 
 int prepare_bounds(const kpm_model *m, int n_sectors, const int32_t *n_up, BoundsLayout *bl) {
-  KPM_TRY(prepare_run(m, n_sectors, n_up, 2, 2, KPM_FP64, &bl->run));
+  // (the plan only: no lists, and no plan of the small-sector kernel)
+  KPM_TRY(prepare_run(m, n_sectors, n_up, 2, 2, KPM_FP64, &bl->run, least_scratch(Knobs())));
   const MomentsRun &r = bl->run;
   bl->list_stride = 0;
   bl->list_estride = 0;

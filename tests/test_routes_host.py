@@ -2,10 +2,12 @@
 import os
 import shutil
 import subprocess
+import time
 
 import pytest
 
 import kpm_workloads as W
+import paper_2104_13218_gb300 as kpm
 from paper_2104_13218_gb300 import _lib
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -81,3 +83,19 @@ def test_fixed_point_keeps_the_lists(route, model):
     (W.ring(12), [6], 1, 1), (W.ring(16), [-1], 100, 1), (W.ladder(16), [8, 9, 10, 11, 12, 13, 14, 15, 16], 1, 1)])
 def test_small_sectors_rule(route, model, n_up, R, one_launch):
     assert route(model, n_up, R)["small"] == one_launch
+
+
+# The bounds need the plan of the states alone: with the plans of a whole space's sectors on top
+# their size query (and call) took five times as long, longer than for a sector of it.
+def test_bounds_prepare_no_more_than_the_plan():
+    model = W.ring(16)
+
+    def shortest(n_up):
+        t = []
+        for _ in range(60):
+            t0 = time.perf_counter()
+            kpm.bounds_workspace_size(model, n_up)
+            t.append(time.perf_counter() - t0)
+        return min(t)
+
+    assert shortest([-1]) < shortest([8])
