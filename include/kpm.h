@@ -212,12 +212,14 @@ size_t kpm_moments_ex_workspace_size(const kpm_model *model, int32_t n_sectors,
  *
  * The paper has no counterpart.  Times short runs of the problem (the random
  * vectors, 1 + trial_steps matrix-vector products and the assembly, best of
- * two, CUDA events on `stream`) for a one-pass coordinate search over: the
- * neighbour-list or the matrix-free step kernel, the states per tile, the
+ * two, CUDA events on `stream`) for a one-pass coordinate search over: small
+ * sectors in one launch or by steps, the neighbour-list or the matrix-free step kernel
+ * (with KPM_FP64 the latter has FP64 vectors in place of fixed-point ones), the states per
+ * tile, the
  * resident blocks per SM, one or two states per warp for FP32 rows of 17..32
  * chunks, and (FP32) the sector dimension below which sectors run in FP64
- * (searched upwards from 1024 only).  None of these changes the arithmetic
- * beyond the order of the sums.  The best choice is kept for the life of the
+ * (searched upwards from 1024 only).  None of these changes the results beyond
+ * rounding.  The best choice is kept for the life of the
  * process, keyed by (model, sectors, R, precision), and used by calls whose
  * kpm_opts.tuned is 1.  a, b: host [n_sectors] rescaling.  Outputs (host, may
  * be NULL): default_ms and best_ms, the measured time per matrix-vector

@@ -1,7 +1,9 @@
 // Autotuner of the moment loop (the paper has no counterpart): a search over
 // the choices that change only the schedule of the Chebyshev step, not its
 // arithmetic beyond the order of the sums:
-//   - neighbour-list, hi-block or matrix-free kernel (where they apply),
+//   - small sectors in one launch or by steps, and the neighbour-list, hi-block or
+//     matrix-free kernel of the steps (where they apply; without lists the FP64 form has FP64
+//     vectors in place of fixed-point ones),
 //   - states per tile,
 //   - resident blocks per SM of the persistent grid,
 //   - FP32 rows of 17..32 chunks as two states per warp or one,
@@ -49,56 +51,100 @@ std::string problem_key(const kpm_model *m, int n_sectors, const int32_t *n_up, 
   return k;
 }
 
-void describe(const Knobs &kn, bool lists, bool block, char *out, size_t len) {
+// What a candidate ran as (of its main run, or of the FP64 side run when that is all).
+struct Ran {
+  bool small = false, lists = false, weighted = false, fixed = false, block = false;
+  int64_t tile_states = 0;
+  int grid = 0, G = 0, cpl = 0, n_sectors = 0;
+  Ran() = default;
+  explicit Ran(const MomentsJob &job) {
+    const MomentsRun &r = job.has_main ? job.main : job.side;
+    small = r.small;
+    weighted = r.weighted;
+    lists = r.list_stride > 0;
+    fixed = r.fixed;
+    block = r.block_L > 0;
+    tile_states = r.plan.tile_states;
+    grid = small ? 0 : r.grid;
+    G = r.lay.G;
+    cpl = r.lay.cpl;
+    n_sectors = r.plan.n_sectors;
+  }
+  // The same run: a knob that changes nothing (a tile above the kernel's most, more
+  // blocks than an SM holds) is not to be chosen by the noise of its time.
+  bool operator==(const Ran &o) const {
+    return small == o.small && lists == o.lists && weighted == o.weighted && fixed == o.fixed &&
+           block == o.block && tile_states == o.tile_states && grid == o.grid && G == o.G &&
+           cpl == o.cpl && n_sectors == o.n_sectors;
+  }
+  const char *kernel() const {
+    if (small) return "small-sector";
+    if (block) return "hi-block";
+    if (weighted) return fixed ? "weighted-list (fixed point)" : "weighted-list";
+    if (lists) return fixed ? "list (fixed point)" : "list";
+    return "matrix-free";
+  }
+};
+
+void describe(const Knobs &kn, const Ran &ran, char *out, size_t len) {
   snprintf(out, len, "kernel=%s tile_states=%lld blocks_per_sm=%d two_state=%d side_min_dim=%lld",
-           block ? "hi-block" : (lists ? "list" : "matrix-free"), (long long)kn.tile_states,
-           kn.blocks_per_sm, kn.two_state, (long long)kn.side_min_dim);
+           ran.kernel(), (long long)kn.tile_states, kn.blocks_per_sm, kn.two_state,
+           (long long)kn.side_min_dim);
 }
 
-// Times one candidate: init, 1 + steps matrix-vector products and assembly.
+// Times one candidate: init, 1 + steps matrix-vector products and assembly.  A
+// candidate that leaves the fixed-point range is timed as the FP64 run that a call would make.
 int time_candidate(const kpm_model *m, int n_sectors, const int32_t *n_up, const double *a,
                    const double *b, int R, int precision, int steps, const Knobs &kn,
-                   cudaStream_t s, double *ms, bool *uses_lists, Knobs *resolved,
-                   bool *uses_block = nullptr) {
+                   cudaStream_t s, double *ms, Ran *ran) {
   MomentsJob job;
   const int K = 2 * (steps + 1);
   KPM_TRY(prepare_job(m, n_sectors, n_up, K, R, precision, &job, kn));
   Workspace ws;
   const size_t out_bytes = align256((size_t)n_sectors * K * sizeof(double));
   KPM_TRY(ws.acquire(nullptr, 0, job_bytes(job) + out_bytes, s));
-  Arena arena{reinterpret_cast<char *>(ws.ptr), ws.size, 0};
-  KPM_TRY(setup_job(job, a, b, arena, s));
-  double *mu = arena.take<double>((size_t)n_sectors * K);
-  KPM_REQUIRE(mu != nullptr, KPM_ENOMEM, "workspace too small");
   cudaEvent_t e0, e1;
   KPM_CUDA(cudaEventCreate(&e0));
   KPM_CUDA(cudaEventCreate(&e1));
-  double best = 1e300;
-  for (int rep = 0; rep < 2; ++rep) {
-    // the counters of the tile queues start at zero for every run
-    for (int part = 0; part < 2; ++part) {
-      MomentsRun *r = part == 0 ? (job.has_main ? &job.main : nullptr)
-                                : (job.has_side ? &job.side : nullptr);
-      if (r) KPM_CUDA(cudaMemsetAsync(r->counters, 0, sizeof(int) * 2 * r->S, s));
+  struct Events {
+    cudaEvent_t a, b;
+    ~Events() {
+      cudaEventDestroy(a);
+      cudaEventDestroy(b);
     }
-    KPM_CUDA(cudaEventRecord(e0, s));
-    KPM_TRY(run_job(job, 1, 0, mu, nullptr, nullptr, s));
-    KPM_CUDA(cudaEventRecord(e1, s));
-    KPM_CUDA(cudaEventSynchronize(e1));
-    float t = 0.f;
-    KPM_CUDA(cudaEventElapsedTime(&t, e0, e1));
-    best = std::min(best, (double)t);
+  } events{e0, e1};
+  MomentsRun *const runs[2] = {job.has_main ? &job.main : nullptr, job.has_side ? &job.side : nullptr};
+  for (;;) {
+    Arena arena{reinterpret_cast<char *>(ws.ptr), ws.size, 0};
+    double *mu = arena.take<double>((size_t)n_sectors * K);
+    KPM_REQUIRE(mu != nullptr, KPM_ENOMEM, "workspace too small");
+    KPM_TRY(setup_job(job, a, b, arena, s));
+    double best = 1e300;
+    for (int rep = 0; rep < 2; ++rep) {
+      // the counters of the tile queues start at zero for every run
+      for (MomentsRun *r : runs)
+        if (r) KPM_CUDA(cudaMemsetAsync(r->counters, 0, sizeof(int) * 2 * r->S, s));
+      KPM_CUDA(cudaEventRecord(e0, s));
+      KPM_TRY(run_job(job, 1, 0, mu, nullptr, nullptr, s));
+      KPM_CUDA(cudaEventRecord(e1, s));
+      KPM_CUDA(cudaEventSynchronize(e1));
+      float t = 0.f;
+      KPM_CUDA(cudaEventElapsedTime(&t, e0, e1));
+      best = std::min(best, (double)t);
+    }
+    *ms = best;
+    *ran = Ran(job);
+    int flags = 0;
+    for (MomentsRun *r : runs) {
+      int f = 0;
+      if (r) KPM_CUDA(cudaMemcpyAsync(&f, r->flag, sizeof(int), cudaMemcpyDeviceToHost, s));
+      KPM_CUDA(cudaStreamSynchronize(s));
+      flags |= f;
+    }
+    if (!(flags & kFlagRange)) return KPM_OK;
+    for (MomentsRun *r : runs)
+      if (r) r->fixed = r->small = false;
   }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  *ms = best;
-  if (uses_lists) *uses_lists = job.has_main && job.main.list_stride > 0;
-  if (uses_block) *uses_block = job.has_main && job.main.block_L > 0;
-  if (resolved) {
-    *resolved = kn;
-    if (job.has_main) resolved->tile_states = job.main.plan.tile_states;
-  }
-  return KPM_OK;
 }
 
 }  // namespace
@@ -129,50 +175,57 @@ extern "C" int kpm_autotune(const kpm_model *model, int32_t n_sectors, const int
   KPM_TRY(validate_sectors(model, n_sectors, n_up));
   Knobs best;
   double t_def = 0.0;
-  bool lists = false;
-  Knobs resolved;
-  KPM_TRY(time_candidate(model, n_sectors, n_up, a, b, R, precision, trial_steps, best, s, &t_def,
-                         &lists, &resolved));
-  const int64_t ts0 = resolved.tile_states;
-  bool uses_block = false;
-  {
-    MomentsJob probe;
-    if (prepare_job(model, n_sectors, n_up, 2, R, precision, &probe) == KPM_OK)
-      uses_block = probe.has_main && probe.main.block_L > 0;
-  }
+  Ran ran;  // of the best choice so far
+  KPM_TRY(time_candidate(model, n_sectors, n_up, a, b, R, precision, trial_steps, best, s, &t_def, &ran));
   double t_best = t_def;
   std::string log;
   char line[256];
   auto consider = [&](const Knobs &cand) -> int {
     double t = 0.0;
-    bool l = false, bk = false;
-    int rc = time_candidate(model, n_sectors, n_up, a, b, R, precision, trial_steps, cand, s, &t,
-                            &l, nullptr, &bk);
-    if (rc == KPM_ENOMEM) return KPM_OK;  // a candidate that does not fit is skipped
+    Ran c;
+    int rc = time_candidate(model, n_sectors, n_up, a, b, R, precision, trial_steps, cand, s, &t, &c);
+    if (rc == KPM_ENOMEM) {  // a candidate that does not fit is skipped
+      clear_error();
+      return KPM_OK;
+    }
     KPM_TRY(rc);
-    describe(cand, l, bk, line, sizeof(line));
+    describe(cand, c, line, sizeof(line));
     log += line;
     snprintf(line, sizeof(line), ": %.4f ms\n", t);
     log += line;
-    if (t < t_best) {
+    if (t < t_best && !(c == ran)) {
       t_best = t;
       best = cand;
+      ran = c;
     }
     return KPM_OK;
   };
   // 1. kernel
-  if (lists) {
+  if (ran.small) {
     Knobs c = best;
-    c.lists = 0;
+    c.small = 0;
     KPM_TRY(consider(c));
   }
-  if (uses_block) {
+  if (!ran.small && ran.weighted) {
+    Knobs c = best;
+    c.weighted = c.small = 0;
+    KPM_TRY(consider(c));
+  }
+  if (!ran.small && ran.lists) {
+    Knobs c = best;
+    c.lists = c.small = 0;
+    KPM_TRY(consider(c));
+  }
+  if (!ran.small && ran.block) {
     Knobs c = best;
     c.block = 0;
     KPM_TRY(consider(c));
   }
+  // the small-sector kernel has neither tiles nor a choice of blocks
+  const int64_t ts0 = ran.tile_states;
+  const bool tiles = !ran.small;
   // 2. states per tile
-  {
+  if (tiles) {
     const Knobs base = best;
     for (int64_t f : {ts0 / 4, ts0 / 2, ts0 * 2, ts0 * 4}) {
       if (f < 1) continue;
@@ -182,7 +235,7 @@ extern "C" int kpm_autotune(const kpm_model *model, int32_t n_sectors, const int
     }
   }
   // 3. resident blocks per SM
-  {
+  if (tiles) {
     const Knobs base = best;
     for (int bps : {1, 2, 3}) {
       Knobs c = base;
@@ -212,14 +265,7 @@ extern "C" int kpm_autotune(const kpm_model *model, int32_t n_sectors, const int
   if (default_ms) *default_ms = t_def / (trial_steps + 1);
   if (best_ms) *best_ms = t_best / (trial_steps + 1);
   if (report && report_len > 0) {
-    bool l_best = false, b_best = false;
-    // the kernel the best choice resolves to
-    MomentsJob job;
-    if (prepare_job(model, n_sectors, n_up, 2, R, precision, &job, best) == KPM_OK) {
-      l_best = job.has_main && job.main.list_stride > 0;
-      b_best = job.has_main && job.main.block_L > 0;
-    }
-    describe(best, l_best, b_best, line, sizeof(line));
+    describe(best, ran, line, sizeof(line));
     std::string out = std::string("best: ") + line + "\n" + log;
     snprintf(report, report_len, "%s", out.c_str());
   }

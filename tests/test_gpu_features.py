@@ -184,3 +184,23 @@ def test_autotune_keeps_the_results(precision, tol):
 def test_fp64_rate_probe():
     r = kpm.fp64_peak()
     assert 0.05 < r["tflops"] < 200.0 and r["ms"] >= 50.0
+
+
+# The search names the kernels that ran, tries the other form of small sectors and of lists with
+# matrix elements, and no schedule for the small-sector kernel, which has none.
+@pytest.mark.parametrize("model,n_up,precision,kernel,other", [
+    (W.ladder(12), [6, 7], "fp64", "small-sector", "list (fixed point)"),
+    (W.random_bonds(16, 32, 3, 0.2, 1.5), [8], "fp64", "weighted-list (fixed point)", "matrix-free"),
+    (W.random_bonds(16, 32, 3, 0.2, 1.5), [8], "fp32", "weighted-list", "matrix-free"),
+    (W.j1j2_chain(16, 1.0, 0.4), [8], "fp64", "list (fixed point)", "matrix-free")])
+def test_autotune_knows_the_kernels(model, n_up, precision, kernel, other):
+    a, b = [30.0] * len(n_up), [0.0] * len(n_up)
+    res = kpm.autotune(model, n_up, a, b, 20, precision=precision, trial_steps=30)
+    best, *lines = res["report"].splitlines()
+    ran = [line.split("kernel=")[1].split(" tile_states")[0] for line in lines]
+    assert ran[0] == other and best.split("kernel=")[1].split(" tile_states")[0] in (kernel, other)
+    if kernel == "small-sector" and kernel in best:
+        assert ran == [other]  # no tiles, no blocks per SM
+    d = kpm.moments(model, n_up, 20, 20, 3, a=a, b=b, precision=precision)
+    t = kpm.moments(model, n_up, 20, 20, 3, a=a, b=b, precision=precision, tuned=True)
+    assert np.abs(d["mu"] - t["mu"]).max() <= (1e-10 if precision == "fp64" else 1e-5)
