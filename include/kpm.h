@@ -38,7 +38,8 @@
  * - Workspace: calls that need device scratch take (workspace, ws_bytes).
  *   With workspace == NULL the library allocates the scratch itself with
  *   a stream-ordered allocation on `stream` and frees it before returning (up to 256 MB
- *   per device stay in a pool of the library's own for the next call); otherwise the
+ *   per device stay in a pool of the library's own for the next call, until
+ *   kpm_release_scratch); otherwise the
  *   region must be device memory of at least the size the matching
  *   *_workspace_size query returns, aligned to 256 bytes.
  * - Streams: `stream` is a cudaStream_t (NULL = legacy default stream).
@@ -114,6 +115,10 @@ int kpm_version(void);
 
 /* Message of the last failing call on this thread ("" if none). */
 const char *kpm_last_error(void);
+
+/* Returns to the current device the memory that the library keeps between calls (see Workspace
+   above; at most 256 MB).  Calls of other threads may be running; what they use stays. */
+int kpm_release_scratch(void);
 
 /* Dimension of a sector: C(n_sites, n_up), or 2^n_sites for n_up = -1; -1 if invalid. */
 int64_t kpm_sector_dim(int32_t n_sites, int32_t n_up);

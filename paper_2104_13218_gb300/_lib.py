@@ -93,6 +93,7 @@ PROTOTYPES = {
                                   P]),
     "kpm_spin_moments": (c_int32, [P, c_int32, P, P, P, c_int32, c_int32, c_uint64, c_uint64,
                                    c_int32, P, P, P, c_int32, P]),
+    "kpm_release_scratch": (c_int32, []),
     "kpm_profile_enable": (c_int32, [c_int32]),
     "kpm_profile_read": (c_int32, [P, P, P]),
 }

@@ -180,6 +180,11 @@ def autotune(model, n_up, a, b, R: int, precision: str = "fp32", trial_steps: in
     return {"default_ms": d_ms.value, "best_ms": b_ms.value, "report": rep.value.decode()}
 
 
+def release_scratch() -> None:
+    """Return the memory that the library keeps between calls to the current device."""
+    check("kpm_release_scratch", lib().kpm_release_scratch())
+
+
 def fp64_peak(stream=None) -> dict:
     """Measured FP64 FMA rate of the current device: dict(tflops, ms)."""
     t = ctypes.c_double(0)

@@ -233,6 +233,8 @@ class PackedUpload {
 constexpr size_t kScratchKeep = (size_t)256 << 20;
 int scratch_alloc(void **p, size_t bytes, cudaStream_t s);
 void scratch_free(void *p, cudaStream_t s);
+// Returns what the current device's pool keeps and no call is using.
+int scratch_release();
 // Unique id of the calling thread's current CUDA context (0 if there is none or
 // the driver cannot tell).
 unsigned long long current_context_id();

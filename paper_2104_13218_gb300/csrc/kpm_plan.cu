@@ -405,6 +405,16 @@ unsigned long long current_context_id() {
   return id;
 }
 
+int scratch_release() {
+  int dev = 0;
+  KPM_CUDA(cudaGetDevice(&dev));
+  if (dev >= kPoolDevices) return KPM_OK;
+  std::lock_guard<std::mutex> lock(g_pool_mutex);
+  if (g_pools[dev] == nullptr || g_pool_ctx[dev] != current_context_id()) return KPM_OK;
+  KPM_CUDA(cudaMemPoolTrimTo(g_pools[dev], 0));
+  return KPM_OK;
+}
+
 int scratch_alloc(void **p, size_t bytes, cudaStream_t s) {
   cudaMemPool_t pool = bytes <= kScratchKeep ? scratch_pool() : nullptr;
   cudaError_t e = pool != nullptr ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s);
@@ -467,6 +477,11 @@ void profile_push(cudaEvent_t start, cudaEvent_t stop) {
 }  // namespace kpm
 
 extern "C" {
+
+int kpm_release_scratch(void) {
+  kpm::clear_error();
+  return kpm::scratch_release();
+}
 
 int kpm_profile_enable(int32_t on) {
   std::lock_guard<std::mutex> lock(kpm::g_prof_mutex);

@@ -89,3 +89,16 @@ def test_gradient_in_a_small_workspace():
             continue
         got, ref = kpm.moments_backward(*args, workspace=ws), kpm.moments_backward(*args)
         assert np.array_equal(got, ref), (a, got, ref)
+
+
+# What the library keeps between calls (up to 256 MB) can be had back, and it works on.
+def test_kept_scratch_is_given_back():
+    model, kw = W.ring(16), dict(a=[6.0], b=[-1.0], device=True)
+    first = kpm.moments(model, [8], 20, 60, 5, **kw)["mu"]
+    kpm.moments(W.ring(18), [9], 10, 100, 5, **kw)  # two vectors of 39 MB
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    kpm.release_scratch()
+    assert torch.cuda.mem_get_info()[0] - before >= 64 << 20
+    kpm.release_scratch()
+    assert torch.equal(kpm.moments(model, [8], 20, 60, 5, **kw)["mu"], first)
