@@ -476,9 +476,9 @@ int kpm_spin_moments(const kpm_spin_model *model, int32_t n_sectors, const int32
 /*
  * Instrumentation (no counterpart in the paper; used by the benchmark).
  * kpm_profile_enable(1) starts recording a CUDA event pair around every
- * launch of the fused Chebyshev step kernel, on the stream it is launched
- * on, and clears earlier records; kpm_profile_enable(0) stops recording.
- * kpm_profile_read waits for the recorded events, returns the summed
+ * launch of the fused Chebyshev step kernel (or of the kernel that makes
+ * all steps of small sectors, one launch), on the stream it is launched on, and
+ * clears earlier records; kpm_profile_enable(0) stops recording.  kpm_profile_read waits for the recorded events, returns the summed
  * device time of the recorded step launches (ms) and their count, and
  * clears the records.  kernel_launches returns the number of kernels the
  * library launched since it was loaded (any pointer may be NULL).

@@ -515,7 +515,18 @@ int launch_small(const MomentsRun &r, uint64_t seed, uint64_t r0, cudaStream_t s
   a.block_sector = m.block_sector;
   a.block_column = m.block_column;
   void *args[] = {(void *)&a};
+  const bool prof = r.profile && profiling();
+  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  if (prof) {
+    KPM_CUDA(cudaEventCreate(&e0));
+    KPM_CUDA(cudaEventCreate(&e1));
+    KPM_CUDA(cudaEventRecord(e0, s));
+  }
   KPM_CUDA(cudaLaunchKernel(fn, dim3(n_blocks), dim3(threads), args, small_smem(D), s));
+  if (prof) {
+    KPM_CUDA(cudaEventRecord(e1, s));
+    profile_push(e0, e1);
+  }
   count_launches(1);
   const int ns = r.plan.n_sectors, per_block = kSumsThreads / 32;
   const int grid = std::min(4096, (r.S * ns + per_block - 1) / per_block);

@@ -416,3 +416,9 @@ def test_abandoned_run_stops():
     fixed, fp64, left = step_ms(30.0), step_ms(30.0, vectors="basis"), step_ms(5.0)
     assert left[1] == fixed[1] + fp64[1] and fp64[0] > 2 * fixed[0]
     assert left[0] < fp64[0] + 0.5 * fixed[0], (fixed, fp64, left)
+
+
+# The launch that makes all products of small sectors is among the recorded step launches.
+def test_small_sector_launch_is_recorded():
+    ms, n = _step_launches(lambda: kpm.moments(W.ring(12), [6], 200, 20, 5, a=[5.0], b=[-1.0]))
+    assert n == 1 and ms > 0.0
