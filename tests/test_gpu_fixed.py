@@ -422,3 +422,41 @@ def test_abandoned_run_stops():
 def test_small_sector_launch_is_recorded():
     ms, n = _step_launches(lambda: kpm.moments(W.ring(12), [6], 200, 20, 5, a=[5.0], b=[-1.0]))
     assert n == 1 and ms > 0.0
+
+
+# ---------------------------------------------------------------- sums of many tiles, runs of parts
+
+# sectors of more tiles than one block sums, with groups and with couplings of their own
+@pytest.mark.parametrize("model", [W.j1j2_chain(20, 1.0, 0.4), W.random_bonds(20, 30, 3, -0.7, 0.7)],
+                         ids=lambda m: m.name)
+def test_sums_in_several_parts(model):
+    bi, bj, J = model.arrays()
+    got = kpm.moments(model, [10], 8, 100, 5, a=[15.0], b=[0.5])
+    # (the oracle adds one product after the other: over all vectors at once it is itself off
+    # by 2.2e-12, mu_0 = 1 - 2.2e-12)
+    ref = np.mean([c_oracle.moments(20, bi, bj, J, 10, 15.0, 0.5, 8, 5, 5, r0)["mu"]
+                   for r0 in range(0, 100, 5)], axis=0)
+    assert np.abs(got["mu"][0] - ref).max() <= 1e-12
+
+
+# a shorter run's moments are the first of a longer run's, bit for bit
+@pytest.mark.parametrize("model,n_up,R", [(W.ladder(12), [6, 7], 20), (W.j1j2_chain(20, 1.0, 0.4), [10], 100),
+                                          (W.random_bonds(18, 30, 3, -0.7, 0.7), [9, 5], 20), (W.ring(17), [-1], 9)])
+def test_shorter_runs_are_prefixes(model, n_up, R):
+    kw = dict(a=[16.0] * len(n_up), b=[0.5] * len(n_up), device=True)
+    short, long_ = (kpm.moments(model, n_up, K, R, 5, **kw) for K in (12, 24))
+    for q in ("mu", "mu_M", "mu_M2"):
+        assert torch.equal(short[q], long_[q][:, :12]), q
+
+
+# FP32 with a large sector, and a small one (in FP64) whose interval is too narrow: both runs are
+# made again, on two streams
+def test_fp32_side_run_outside_the_interval():
+    model, n_up, a, b = W.ring(16), [8, 2], [6.0, 1.0], [-1.0, 3.0]
+    got = kpm.moments(model, n_up, K, 20, 5, a=a, b=b, precision="fp32", allow_ebounds=True)
+    assert got["status"] == 6
+    bi, bj, J = model.arrays()
+    refs = [c_oracle.moments(16, bi, bj, J, k, a[i], b[i], K, 20, 5)["mu"] for i, k in enumerate(n_up)]
+    assert np.abs(got["mu"][0] - refs[0]).max() <= 1e-5
+    scale = np.abs(refs[1]) + 1e-12 * np.abs(refs[1]).max()
+    assert (np.abs(got["mu"][1] - refs[1]) <= 1e-9 * scale).all()

@@ -102,3 +102,16 @@ def test_kept_scratch_is_given_back():
     assert torch.cuda.mem_get_info()[0] - before >= 64 << 20
     kpm.release_scratch()
     assert torch.equal(kpm.moments(model, [8], 20, 60, 5, **kw)["mu"], first)
+
+
+# A problem whose default scratch exceeds the static array and whose least does not.
+def test_static_scratch_takes_the_least_form():
+    model, n_up, K, R = W.random_bonds(19, 38, 3, -0.7, 0.7), [9], 12, 10
+    assert kpm.moments_workspace_size(model, n_up, K, R, "fp64") > kpm.lib().kpm_static_scratch_bytes()
+    a, b, nu = np.array([16.0]), np.array([0.5]), np.array(n_up, dtype=np.int32)
+    mu = torch.full((1, K), float("nan"), dtype=torch.float64, device="cuda")
+    rc = kpm.lib().kpm_moments_static(kpm.CModel.of(model).ref, 1, nu.ctypes.data, a.ctypes.data, b.ctypes.data, K, R,
+                                      5, 0, 0, mu.data_ptr(), None, None, torch.cuda.current_stream().cuda_stream)
+    assert rc == 0
+    ref = kpm.moments(model, n_up, K, R, 5, a=a, b=b)["mu"]
+    assert np.abs(mu.cpu().numpy() - ref).max() <= 1e-10
