@@ -705,10 +705,12 @@ bool fixed_spin_couplings(const kpm_spin_model *m, const SpinPlan &p, const doub
     const FxPair A = fx_two_over(a[i]);
     FxPair d = fx_pair_mul(A, fx_pair_add(top, -b[i]));
     if (p.dim[i] == 1) {
-      // one state: no couplings, and b is this sum in FP64 while a may be tiny
+      // one state: no couplings; in the interval that kpm_spin_bounds gives it b is this sum
+      // in FP64
       double diag = 0.0;
       for (int k = 0; k < m->n_bonds; ++k) diag += m->J[k] * s * s;
-      d = FxPair{2.0 * (1.0 / a[i]) * (diag - b[i]), 0.0};
+      if (a[i] <= kFxPointInterval * std::max(1.0, std::fabs(b[i])))
+        d = FxPair{2.0 * (1.0 / a[i]) * (diag - b[i]), 0.0};
     } else {
       for (int k = 0; k < m->n_bonds; ++k) {
         const FxPair c = fx_pair_mul(A, FxPair{0.5 * m->J[k], 0.0});

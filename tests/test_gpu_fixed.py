@@ -460,3 +460,20 @@ def test_fp32_side_run_outside_the_interval():
     assert np.abs(got["mu"][0] - refs[0]).max() <= 1e-5
     scale = np.abs(refs[1]) + 1e-12 * np.abs(refs[1]).max()
     assert (np.abs(got["mu"][1] - refs[1]) <= 1e-9 * scale).all()
+
+
+# A sector of one state has the moments cos(n arccos x), x = (E - b)/a, without an average over
+# states: an x that is off by d moves mu_n by n d / sqrt(1 - x^2).  x is rounded to 2^-60; the vector's
+# roundings of 0.29/U in the root mean square (U = 2^54 - 1 for 9 bonds) add up to 1.2 sqrt(n) times
+# that after n products, and mu_2n = 2 v_n^2 - 1 to four times that (six standard deviations).
+def test_sector_of_one_state():
+    n, J, a, b, K = 9, 1.0077, 3.0917, 0.5931, 800
+    got = kpm.moments(W.ring(n, J), [n], K, 3, 5, a=[a], b=[b])["mu"][0]
+    L = np.longdouble
+    x = (L(J) * n / 4 - L(b)) / L(a)
+    assert 1 / np.sqrt(1 - x * x) < 1.2
+    t = [L(1), x]
+    for _ in range(K - 2):
+        t.append(2 * x * t[-1] - t[-2])
+    tol = 1.2 * K * 2.0 ** -60 + 6 * 4 * 1.2 * np.sqrt(K / 2) * 0.29 * 2.0 ** -54
+    assert np.abs(got - np.array(t)).max() <= tol
