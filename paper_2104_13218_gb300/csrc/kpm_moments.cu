@@ -1837,6 +1837,7 @@ int launch_step(const MomentsRun &r, const void *x, void *zy, int first, int ste
   a.partials = r.partials;
   a.sums = r.sums + (size_t)step * r.plan.n_sectors * r.NQ;
   a.queue = r.counters + 2 * step;
+  int *next_queue = step + 1 < r.S ? r.counters + 2 * (step + 1) : nullptr;
   a.done = r.counters + 2 * step + 1;
   a.Rp = r.lay.Rp;
   a.G = r.lay.G;
@@ -1893,10 +1894,10 @@ int launch_step(const MomentsRun &r, const void *x, void *zy, int first, int ste
   }
   if (r.weighted)
     KPM_TRY(launch_weighted_step(r.wr, r.precision, r.grid, x, zy, first, a.partials,
-                                 a.prev_partials, a.prev_sums, a.sum_parts, a.queue, s));
+                                 a.prev_partials, a.prev_sums, a.sum_parts, a.queue, next_queue, s));
   else if (r.fixed)
     KPM_TRY(launch_fixed_step(r, x, zy, first, a.partials, a.prev_partials, a.prev_sums, a.sum_parts,
-                              a.queue, step_smem(r), s));
+                              a.queue, next_queue, step_smem(r), s));
   else
     KPM_CUDA(cudaLaunchKernel(fn, dim3(r.grid), dim3(kThreads), args, step_smem(r), s));
   count_launches(1);

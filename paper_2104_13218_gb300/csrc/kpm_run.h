@@ -254,6 +254,6 @@ void fixed_tables(const BondsDev &bd, const std::vector<int64_t> &couplings,
 void *fixed_kernel_ptr(int cpl, bool full);
 int launch_fixed_step(const MomentsRun &run, const void *x, void *zy, int first, double *partials,
                       const double *prev_partials, double *prev_sums, int sum_parts, int *queue,
-                      size_t smem, cudaStream_t s);
+                      int *next_queue, size_t smem, cudaStream_t s);
 
 }  // namespace kpm

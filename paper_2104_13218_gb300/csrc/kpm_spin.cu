@@ -1008,7 +1008,8 @@ int spin_moments_run(const kpm_spin_model *model, int32_t n_sectors, const int32
       part = partials + (step & 1) * slot;
       KPM_TRY(launch_weighted_step(r.wr, precision, grid, x, zy, step == 0, part,
                                    partials + ((step + 1) & 1) * slot,
-                                   step > 0 ? out - (size_t)n_sectors * r.NQ : nullptr, 1, queues + step, s));
+                                   step > 0 ? out - (size_t)n_sectors * r.NQ : nullptr, 1, queues + step,
+                                   step + 1 < S ? queues + step + 1 : nullptr, s));
       count_launches(1);
     } else {
       sa.x = x;

@@ -56,6 +56,6 @@ size_t weighted_smem(const WeightedRun &r);
 void *weighted_kernel_ptr(const WeightedRun &r, int precision);
 int launch_weighted_step(const WeightedRun &r, int precision, int grid, const void *x, void *zy,
                          int first, double *partials, const double *prev_partials,
-                         double *prev_sums, int sum_parts, int *queue, cudaStream_t s);
+                         double *prev_sums, int sum_parts, int *queue, int *next_queue, cudaStream_t s);
 
 }  // namespace kpm
