@@ -925,6 +925,16 @@ inline int sum_parts(const MomentsRun &r) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(64, slots / ((int64_t)r.plan.n_sectors * 2048)));
 }
 
+// Which sums of the steps n > 0 are the moments already: 2 <v_n|v_n> - <v_0|v_0> (fixed-point
+// lists), and 2 <v_{n+1}|v_n> - <v_1|v_0> (small sectors).
+enum Subtracted { kSubtractedNone = 0, kSubtractedEven = 1, kSubtractedBoth = 2 };
+inline int subtracted_sums(const MomentsRun &r) {
+  return r.small ? kSubtractedBoth : r.fixed ? kSubtractedEven : kSubtractedNone;
+}
+__device__ __forceinline__ bool is_moment(int subtracted, int step, bool odd) {
+  return step == 0 || subtracted == kSubtractedBoth || (subtracted == kSubtractedEven && !odd);
+}
+
 // ---------------------------------------------------------------- per-vector moments
 // The moments of each random vector separately, mu^(r)_n = <r|T_n(H')|r>
 // (the terms of the average in Eq. E-2-7), for realisation statistics and
@@ -939,9 +949,10 @@ struct ColArgs {
   double *part;           // [n_chunks][R][2]
   int R, Rp;
   const SectorDev *sectors;
+  int64_t unit;  // fixed point: U
 };
 
-// The same from fixed-point rows: exact integer sums.
+// The same from fixed-point rows: exact integer sums (of 2 |v_n|^2 - |v_0|^2 as in the steps).
 __global__ void __launch_bounds__(kThreads)
     column_dots_fixed_kernel(const __grid_constant__ ColArgs a) {
   __shared__ i128 s_xx[kThreads], s_yx[kThreads];
@@ -956,6 +967,7 @@ __global__ void __launch_bounds__(kThreads)
   for (int c0 = 0; c0 < a.R; c0 += cols) {
     const int col = c0 + cl;
     i128 xx = 0, yx = 0;
+    const i128 start = (i128)a.unit * a.unit;
     if (rl < nl && col < a.R) {
       for (int64_t r0 = r_begin + rl; r0 < r_end; r0 += 16 * nl) {
         FxDot dx, dy;
@@ -963,12 +975,13 @@ __global__ void __launch_bounds__(kThreads)
         for (int k = 0; k < 16; ++k) {
           const int64_t row = r0 + k * nl;
           if (row < r_end) {
+            xx -= start;
             const FxLimbs xv = fx_split(x[row * a.Rp + col]), yv = fx_split(y[row * a.Rp + col]);
             dx.square(xv);
             dy.product(xv, yv);
           }
         }
-        xx += dx.square_value();
+        xx += 2 * dx.square_value();
         yx += dy.product_value();
       }
     }
@@ -1056,7 +1069,7 @@ __global__ void assemble_r_kernel(const __grid_constant__ AssembleRArgs a) {
     const int step = n / 2, q = n & 1;
     const double raw = a.sums_r[(((int64_t)step * a.n_sectors + sec) * a.R + r) * 2 + q];
     const double base = a.sums_r[((int64_t)sec * a.R + r) * 2 + q];  // mu_0 or mu_1 of vector r
-    const double val = step == 0 || a.subtracted ? raw : 2.0 * raw - base;
+    const double val = is_moment(a.subtracted, step, q) ? raw : 2.0 * raw - base;
     a.mu_r[((int64_t)a.sectors[sec].out_index * a.R + r) * a.K + n] = val;
   }
 }
@@ -1136,7 +1149,7 @@ struct AssembleArgs {
   double *mu, *mu_M, *mu_M2;
   int *flag;
   int n_sectors, K, NQ;
-  int subtracted;  // the sums of the later steps are 2 <v_n|v_n> - <v_0|v_0> already
+  int subtracted;  // Subtracted
   double inv_R;
 };
 
@@ -1155,7 +1168,7 @@ __global__ void assemble_kernel(const __grid_constant__ AssembleArgs a) {
       if (full || q == 0) {
         const int qq = 2 * q + (odd ? 1 : 0);
         const double raw = a.sums[((int64_t)step * a.n_sectors + sec) * a.NQ + qq] * a.inv_R;
-        if (step == 0 || a.subtracted) {
+        if (is_moment(a.subtracted, step, odd)) {
           val = raw;
         } else {
           const double base = a.sums[(int64_t)sec * a.NQ + qq] * a.inv_R;  // mu_0 or mu_1
@@ -1166,7 +1179,7 @@ __global__ void assemble_kernel(const __grid_constant__ AssembleArgs a) {
         const int qq = odd ? 1 : 0;
         const double raw = a.sums[((int64_t)step * a.n_sectors + sec) * a.NQ + qq] * a.inv_R;
         const double base = a.sums[(int64_t)sec * a.NQ + qq] * a.inv_R;
-        const double m0 = step == 0 || a.subtracted ? raw : 2.0 * raw - base;
+        const double m0 = is_moment(a.subtracted, step, odd) ? raw : 2.0 * raw - base;
         const double M = a.sectors[sec].Mval;
         val = (q == 1 ? M : M * M) * m0;
       }
@@ -1935,6 +1948,7 @@ int launch_column_dots(const MomentsRun &r, const void *x, const void *y, int st
   a.R = r.lay.R;
   a.Rp = r.lay.Rp;
   a.sectors = r.tb.sectors;
+  a.unit = r.fx_unit;
   if (r.fixed)
     column_dots_fixed_kernel<<<r.n_cd, kThreads, 0, s>>>(a);
   else if (r.precision == KPM_FP32)
@@ -1961,7 +1975,7 @@ int launch_assemble(const MomentsRun &r, double *mu, double *mu_M, double *mu_M2
     ar.n_sectors = r.plan.n_sectors;
     ar.K = r.K;
     ar.R = r.lay.R;
-    ar.subtracted = r.small;
+    ar.subtracted = subtracted_sums(r);
     const int64_t tot = (int64_t)r.plan.n_sectors * r.lay.R * r.K;
     assemble_r_kernel<<<(int)std::min<int64_t>(4096, (tot + 255) / 256), 256, 0, s>>>(ar);
     KPM_CUDA(cudaGetLastError());
@@ -1977,7 +1991,7 @@ int launch_assemble(const MomentsRun &r, double *mu, double *mu_M, double *mu_M2
   a.n_sectors = r.plan.n_sectors;
   a.K = r.K;
   a.NQ = r.NQ;
-  a.subtracted = r.small;
+  a.subtracted = subtracted_sums(r);
   a.inv_R = 1.0 / r.lay.R;
   const int total = r.plan.n_sectors * r.K;
   assemble_kernel<<<(total + 255) / 256, 256, 0, s>>>(a);

@@ -583,7 +583,7 @@ __global__ void __launch_bounds__(kThreads)
 // mu[out][n] (and mu_M, mu_M2) from the per-step sums, as in the spin-1/2 loop.
 __global__ void spin_assemble_kernel(const double *sums, const SpinSectorDev *sectors, double *mu,
                                      double *mu_M, double *mu_M2, int *flag, int n_sectors, int K,
-                                     int NQ, double inv_R) {
+                                     int NQ, double inv_R, int subtracted) {
   const int total = n_sectors * K;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
     const int sec = i / K, n = i - sec * K;
@@ -595,7 +595,8 @@ __global__ void spin_assemble_kernel(const double *sums, const SpinSectorDev *se
       const int qq = (full ? 2 * q : 0) + odd;
       const double raw = sums[((int64_t)step * n_sectors + sec) * NQ + qq] * inv_R;
       const double base = sums[(int64_t)sec * NQ + qq] * inv_R;
-      double val = step == 0 ? raw : 2.0 * raw - base;
+      // (fixed point: the even sums of the later steps are the moments already)
+      double val = step == 0 || (subtracted && !odd) ? raw : 2.0 * raw - base;
       if (!full && q > 0) val *= q == 1 ? sectors[sec].Mval : sectors[sec].Mval * sectors[sec].Mval;
       out[(int64_t)sectors[sec].out_index * K + n] = val;
       if (q == 0 && !(fabs(val) <= 1.0 + 1e-6)) atomicOr(flag, 1);
@@ -1028,7 +1029,7 @@ int spin_moments_run(const kpm_spin_model *model, int32_t n_sectors, const int32
     std::swap(x, zy);
   }
   spin_assemble_kernel<<<(int)std::min<size_t>(4096, (SK + 255) / 256), 256, 0, s>>>(
-      sums, r.tb.sectors, dmu, dmuM, dmuM2, flag, n_sectors, n_moments, r.NQ, 1.0 / R);
+      sums, r.tb.sectors, dmu, dmuM, dmuM2, flag, n_sectors, n_moments, r.NQ, 1.0 / R, r.fixed);
   KPM_CUDA(cudaGetLastError());
   count_launches(2);
   if (!on_device) {

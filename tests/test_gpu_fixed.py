@@ -477,3 +477,34 @@ def test_sector_of_one_state():
         t.append(2 * x * t[-1] - t[-2])
     tol = 1.2 * K * 2.0 ** -60 + 6 * 4 * 1.2 * np.sqrt(K / 2) * 0.29 * 2.0 ** -54
     assert np.abs(got - np.array(t)).max() <= tol
+
+
+# The even moments have no common offset: 2 <v_n|v_n> - <v_0|v_0> is formed before it is rounded
+# (rounded by itself, <v_0|v_0> leaves up to 1e-16, the same for all vectors).  The vectors' own
+# roundings move mu_2n by 4 sqrt(n) 0.29/(U sqrt(D R)), 1.3e-17 at most here (U > 2^53, D R > 2000), and
+# their mean over 29 moments by a fifth of that; six standard deviations.
+@pytest.mark.parametrize("Q,R", [(8, 7), (9, 5), (10, 4), (11, 6), (12, 3), (13, 5)])
+def test_even_moments_have_no_offset(Q, R):
+    n, two_s, J, a, b, K = 5, 5, 1.0073, 40.1237, -6.4931, 60
+    L = np.longdouble
+    rank = np.arange(6 ** n)
+    q = np.stack([(rank // 6 ** i) % 6 for i in range(n)])
+    codes = sum(q[i].astype(np.int64) << (3 * i) for i in range(n))
+    order = np.argsort(codes)
+    order = order[q.sum(0)[order] == Q]
+    codes, q = codes[order], q[:, order]
+    where = {int(c): k for k, c in enumerate(codes)}
+    diag, rows, cols, vals = np.zeros(len(codes), L), [], [], []
+    for i in range(n):
+        j = (i + 1) % n
+        diag += L(J) / 4 * ((2 * q[i] - two_s) * (2 * q[j] - two_s))
+        for p, r in ((i, j), (j, i)):
+            k = (two_s - q[p]) * (q[p] + 1) * q[r] * (two_s - q[r] + 1)
+            ok = np.nonzero(k > 0)[0]
+            rows.append(ok)
+            cols.append(np.array([where[int(c)] for c in codes[ok] + (1 << 3 * p) - (1 << 3 * r)]))
+            vals.append(L(J) / 2 * np.sqrt(k[ok].astype(L)))
+    ref = _extended(codes, diag, np.concatenate(rows), np.concatenate(cols), np.concatenate(vals), a, b, K, R, 5,
+                    np.zeros(len(codes), L))[0]
+    got = kpm.spin_moments(W.ring(n, J), two_s, [Q], K, R, 5, [a], [b])["mu"][0]
+    assert len(codes) * R > 2000 and abs((got - ref)[2::2].mean()) <= 6 * 1.3e-17 / 5
