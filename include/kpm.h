@@ -40,8 +40,11 @@
  *   a stream-ordered allocation on `stream` and frees it before returning (up to 256 MB
  *   per device stay in a pool of the library's own for the next call, until
  *   kpm_release_scratch); otherwise the
- *   region must be device memory of at least the size the matching
- *   *_workspace_size query returns, aligned to 256 bytes.
+ *   region must be device memory aligned to 256 bytes, of the size the matching
+ *   *_workspace_size query returns.  Where less is given, or the library cannot allocate as
+ *   much, moments, gradients and spin moments are made with the kernels that need the
+ *   least scratch, if that fits: slower, with results that agree to rounding.  For models with
+ *   many different couplings the difference is up to 16 bytes per state and neighbour.
  * - Streams: `stream` is a cudaStream_t (NULL = legacy default stream).
  *   Every call enqueues its work on that stream, then waits for it, and
  *   returns a status; results are complete when the call returns.
@@ -70,10 +73,10 @@ extern "C" {
 #define KPM_EBOUNDS 6   /* |mu_n| > 1 + 1e-6: the spectrum of H' left [-1, 1]; results are written */
 
 /* vector storage precision of the moment loop */
-#define KPM_FP64 0      /* vectors and arithmetic in FP64, or (random signs; sectors of at most
-                           13500 states, or 3 <= R <= 128) in 64-bit fixed point of that
-                           precision; a run whose components leave its range, as with a
-                           spectrum outside [-1, 1], is made in FP64 */
+#define KPM_FP64 0      /* vectors and arithmetic in FP64, or in 64-bit fixed point that rounds no
+                           more (random signs; up to some 50 equal or 100 different bonds; 3 to
+                           128 vectors, or small sectors); a run whose components leave its
+                           range, as with a spectrum outside [-1, 1], is made in FP64 */
 #define KPM_FP32 1      /* vectors and arithmetic in FP32, dot products reduced in FP64;
                            sectors below 1024 states are stored in FP64 (in such tiny
                            sectors FP32 rounding stays coherent and grows with the order) */
@@ -355,7 +358,9 @@ int kpm_realisations(int32_t n_sectors, int32_t n_moments, int32_t R, int32_t R_
  * checkpoint (a run in fixed point, see KPM_FP64, whose coupling groups each
  * lie in one class regenerates them exactly and stores none), and accumulates dL/dJ_b = (1/R) [sum_n (2/a) <lambda_{n+1}, H_b v_n>
  * + (1/a) <lambda_1, H_b v_0>] (dot products over all R vectors).  FP64 only (precision must be KPM_FP64).
- * Workspace: kpm_moments_backward_workspace_size.
+ * Workspace: kpm_moments_backward_workspace_size, which counts the stored pairs; a run in
+ * fixed point does without them, and needs them (else KPM_ENOMEM) only where it
+ * leaves the range and is made again in FP64.
  */
 int kpm_moments_backward(const kpm_model *model, const int32_t *bond_class, int32_t n_classes,
                          int32_t n_sectors, const int32_t *n_up, const double *a,
@@ -398,8 +403,9 @@ int kpm_moments_backward_ex(const kpm_model *model, const int32_t *bond_class, i
  *   a, b         -- host [n_sectors] rescaling (required: no bound estimate is run).
  *   mu, mu_M, mu_M2 -- DEVICE arrays [n_sectors][K] (mu_M, mu_M2 may be NULL).
  *   other arguments as in kpm_moments.
- * Returns KPM_ENOMEM, with the needed size in kpm_last_error(), when the
- * problem's scratch (kpm_moments_workspace_size) exceeds the array.  The
+ * Where the problem's scratch (kpm_moments_workspace_size) exceeds the array, the kernels that
+ * need the least are taken; returns KPM_ENOMEM, with that size in kpm_last_error(), when
+ * theirs does, too.  The
  * first call on a device looks up the array's device address with
  * cudaGetSymbolAddress while that device is current (and so does the first
  * call after the device's context was replaced, e.g. by cudaDeviceReset).

@@ -1347,7 +1347,7 @@ int prepare_run(const kpm_model *m, int n_sectors, const int32_t *n_up, int K, i
       return stride;
     };
     const RowLayout single = run->lay;
-    if (run->fixed && KPM_FIXED_PAIR && run->lay.cpl == 1 && run->lay.G % 2 == 0 && run->lay.G >= 4) {
+    if (run->fixed && run->lay.cpl == 1 && run->lay.G % 2 == 0 && run->lay.G >= 4) {
       // two chunks per lane (one 32-byte load), twice the states per warp: 2 to 10%
       // faster than one chunk (J1-J2 chain N = 18, R = 32; ladder N = 16, R = 100)
       run->lay.cpl = 2;

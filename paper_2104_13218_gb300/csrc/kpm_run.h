@@ -237,9 +237,6 @@ int launch_small(const MomentsRun &r, uint64_t seed, uint64_t r0, cudaStream_t s
 #ifndef KPM_FIXED_BATCH
 #define KPM_FIXED_BATCH 12  // chunks per lane and batch
 #endif
-#ifndef KPM_FIXED_PAIR
-#define KPM_FIXED_PAIR 1  // rows of an even number of chunks: two chunks per lane
-#endif
 __host__ __device__ constexpr int fixed_batch(int cpl) { return KPM_FIXED_BATCH / cpl; }
 int64_t fixed_unit(const BondsDev &b);
 // Coefficients of 2H/a and 2(H - b)/a in units of 2^-59: per sector J/a of every group

@@ -2,9 +2,9 @@
 their layouts and of their range.
 
 Tolerance of moments within the spectral interval: 1e-12, a hundred times below the FP64
-tolerance of the parity tests.  A component is rounded to U/sqrt(D) 2^-1 with
-U >= 2^49 (255 bonds), so a step adds at most 2^-50 of the vector's norm, and
-n steps at most n^2 2^-50 to mu_n: 2e-13 at n = 15 matrix-vector products."""
+tolerance of the parity tests.  A component is rounded by at most 1/(2 U sqrt(D)) with
+U > 2^52, so a step adds at most 2^-53 of the vector's norm, and n steps at most
+n^2 2^-52 to mu_n: 5e-14 at n = 15 matrix-vector products."""
 import ctypes
 
 import numpy as np
