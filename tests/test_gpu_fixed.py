@@ -508,3 +508,31 @@ def test_even_moments_have_no_offset(Q, R):
                     np.zeros(len(codes), L))[0]
     got = kpm.spin_moments(W.ring(n, J), two_s, [Q], K, R, 5, [a], [b])["mu"][0]
     assert len(codes) * R > 2000 and abs((got - ref)[2::2].mean()) <= 6 * 1.3e-17 / 5
+
+
+# Coefficients within the range and levels outside [-1, 1]: the components leave the range during
+# the run, which is given up and made again in FP64 (small sectors and whole space, lists,
+# bonds of their own in both; gradient and spin s below).
+@pytest.mark.parametrize("model,n_up,R,a", [
+    (W.ring(12), [4, 6, -1], 9, 3.6), (W.ring(16), [8], 9, 4.8), (W.ring(17), [-1], 5, 5.1), (_bonds(10, 23), [5, -1], 9, 1.6),
+    (_bonds(17, 34), [8], 9, 2.4)], ids=lambda v: getattr(v, "name", None))
+def test_components_leave_the_range(model, n_up, R, a):
+    bi, bj, J = model.arrays()
+    b = 0.0 if model.name.startswith("ring") else 0.25 * float(np.sum(J))
+    got = kpm.moments(model, n_up, K, R, 5, a=[a] * len(n_up), b=[b] * len(n_up), allow_ebounds=True)
+    assert got["status"] == 6
+    for i, k in enumerate(n_up):
+        ref = c_oracle.moments(model.n_sites, bi, bj, J, k, a, b, K, R, 5)
+        for q in ref:
+            scale = np.abs(ref[q]) + np.abs(ref[q]).max() * 1e-12
+            assert (np.abs(got[q][i] - ref[q]) <= 1e-9 * scale).all(), (k, q)
+
+
+def test_gradient_components_leave_the_range():
+    got, ref, size = _gradient(8, 40, 1.0, a=3.5, ckpt=2)
+    assert (np.abs(got - ref) <= 1e-9 * size).all(), (got, ref)
+
+
+def test_spin_components_leave_the_range():
+    got = _check_spin(3, 5, [7, -1], 5, 6.0, 0.0, 1e-9, "fp64")
+    assert got["status"] == 6
