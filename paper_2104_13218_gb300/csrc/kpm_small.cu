@@ -194,6 +194,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) small_run_kernel(const __gri
   }
   __syncthreads();
   unsigned top = 0;
+  const int flag = threadIdx.x == 0 ? __ldcg(a.flag) & kFlagRange : 0;
   i128 *out = a.part + ((size_t)sec * a.R + col) * a.S * 2;
   for (int n = 0; n < a.S; ++n) {
     FxDot xx, yx;
@@ -248,10 +249,10 @@ __global__ void __launch_bounds__(kSmallThreads, 1) small_run_kernel(const __gri
       const i128 v = warp_sums<2>(acc);
       if ((lane & 15) == 0) slot[(lane >> 4) * 32 + warp] = v;
     }
-    // a run that left the range ends (its results are not used): looked at every 16 steps
+    // a vector that left the range ends (the run's results are not used): looked at every 16
+    // steps, and after the first one whether the coefficients had left it
     if ((n & 15) == 0) {
-      const bool out = top >= 2 * a.lim_hi || (threadIdx.x == 0 && (__ldcg(a.flag) & kFlagRange));
-      if (__syncthreads_or(out)) break;
+      if (__syncthreads_or(top >= 2 * a.lim_hi || (n == 0 && flag != 0))) break;
     } else {
       __syncthreads();
     }
